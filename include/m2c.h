@@ -203,9 +203,10 @@ m2c_status m2c_set_riemann_start(m2c_ctx* ctx, int fp32_start);
  * columns marching tile_z cells along z (0: automatic). M2C_FP64 results do
  * not depend on the tiling (bitwise); M2C_MIXED results agree to FP32 rounding
  * (FP32 multiply-adds may be contracted differently in the code that opens a
- * z-chunk and in the kernels of other tile heights). Default: 16 rows for
- * M2C_MIXED grids large enough to give every SM 8 tiles of 16 rows and 16
- * planes, else 8. */
+ * z-chunk and in the kernels of other tile heights). Default: the
+ * rows (8, or 16 for M2C_MIXED and 4 for M2C_FP64) and tile_z with the smaller
+ * estimated time for the grid's size: short tiles that give every SM work on a
+ * small grid, longer ones on a large grid. */
 m2c_status m2c_set_tiling(m2c_ctx* ctx, int tile_rows, int tile_z);
 
 /* Borrows the device arrays W (5N doubles, the conserved state of Sec. 3.2,

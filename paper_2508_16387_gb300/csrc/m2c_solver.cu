@@ -755,6 +755,7 @@ void set_tiling(Grid& g, int ty, int tz) {
   g.tiles_y = (g.ny + ty - 1) / ty;
   g.tz = std::max(1, std::min(tz, g.nz));
   g.tiles_z = (g.nz + g.tz - 1) / g.tz;
+  g.tz = (g.nz + g.tiles_z - 1) / g.tiles_z;  // the same number of chunks, evenly
 }
 
 long long ntiles_of(const Grid& g) { return (long long)g.tiles_x * g.tiles_y * g.tiles_z; }
@@ -769,24 +770,77 @@ m2c_status push_grid(m2c_ctx* c) {
   return cuda_check(c, e, "descriptor upload");
 }
 
-// Default tile z-chunk: 64, 32 or 16 planes, the longest that still gives the
-// SMs 16 tiles each (the z warm-up of a chunk costs about four planes of
-// loads); short grids take one chunk.
-// Default tile rows: 16 on the mixed path when 16-row tiles of 16 planes
-// still give every SM 8 of them (measured ~3 % faster than 8 rows at 256^3),
-// else 8.
-int default_rows(const Grid& g) {
-  if (g.prec != M2C_MIXED) return 8;
-  const long long tiles16 = (long long)((g.nx + 31) / 32) * ((g.ny + 15) / 16) * ((g.nz + 15) / 16);
-  return tiles16 >= 8ll * sm_count() ? 16 : 8;
+// Tiling of the bulk kernel. A tile marches tz planes and spends about kOpen
+// planes' time on opening its z window, so long tiles waste least; short ones
+// spread a small grid over the SMs and even out tiles of unequal cost (a
+// locally uniform plane is cheaper). Estimated launch time in plane times of one
+// resident block: below one tile per slot the tiles run side by side, the most
+// loaded SM sets the time; above, the tiles' planes over the slots plus half a
+// tile of tail. slots = resident blocks x SMs; t1 and tR are the times of a
+// plane with one and with all `blocks` of them on the SM: a plane takes 14 us
+// alone and 17-20 us beside three others in the mixed kernel (8 rows; latency
+// bound), and as long as the FP64 pipe needs in the FP64 kernel. Measured per
+// launch with the former fixed 16-plane chunks and now: 48^3 mixed 242 -> 38 us,
+// 131x67x45 mixed 381 -> 120, 112^3 mixed 281 -> 201, 192^3 mixed 1184 -> 1021
+// (16 rows), 128x4x4 FP64 207 -> 55, 128^3 FP64 2795 -> 2664.
+struct TileShape {
+  int rows, blocks;
+  double t1, tR;
+};
+constexpr double kOpen = 1.2;
+
+// Tiles of n grids at `rows` rows and a chunk of at most tz planes.
+long long tiles_at(const Grid* const* g, int n, int rows, int tz) {
+  long long t = 0;
+  for (int i = 0; i < n; ++i)
+    t += (long long)((g[i]->nx + 31) / 32) * ((g[i]->ny + rows - 1) / rows) * ((g[i]->nz + tz - 1) / tz);
+  return t;
+}
+
+double launch_estimate(const TileShape& s, long long tiles, int tz) {
+  const double sms = sm_count(), slots = sms * s.blocks, len = tz + kOpen;
+  const double k = std::ceil(tiles / sms);
+  const double t = s.blocks > 1 ? s.t1 + (s.tR - s.t1) * (std::min<double>(k, s.blocks) - 1) / (s.blocks - 1) : s.t1;
+  return tiles <= slots ? 1.7 * t * len : s.tR * (tiles * len / slots + 0.75 * len);
+}
+
+// Chunk length (at most 64 planes) with the smallest estimate for the grids of one launch.
+int choose_tz(const Grid* const* g, int n, const TileShape& s, double* best_out = nullptr) {
+  int zmax = 1, best_tz = 1;
+  for (int i = 0; i < n; ++i) zmax = std::max(zmax, g[i]->nz);
+  double best = INFINITY;
+  for (int tz = 1; tz <= std::min(zmax, 64); ++tz) {
+    const double e = launch_estimate(s, tiles_at(g, n, s.rows, tz), tz);
+    if (e < best) {
+      best = e;
+      best_tz = tz;
+    }
+  }
+  if (best_out) *best_out = best;
+  return best_tz;
+}
+
+TileShape tile_shape(int prec, int rows) {
+  if (prec == M2C_FP64) return rows == 4 ? TileShape{4, 2, 0.75, 1.05} : TileShape{8, 1, 1.0, 1.0};
+  if (rows == 16) return TileShape{16, 2, 15.5, 17.5};
+  return rows == 4 ? TileShape{4, 6, 14.0, 18.0} : TileShape{8, 4, 14.0, 19.0};
 }
 
 int default_tz(const Grid& g, int ty) {
-  const long long cols = (long long)((g.nx + 31) / 32) * ((g.ny + ty - 1) / ty);
-  const long long want = 16ll * sm_count();
-  for (int tz : {64, 32})
-    if (g.nz > tz && cols * ((g.nz + tz - 1) / tz) >= want) return tz;
-  return g.nz > 16 ? 16 : g.nz;
+  const Grid* one[1] = {&g};
+  return choose_tz(one, 1, tile_shape(g.prec, ty));
+}
+
+// Tile rows: 8, or the other shape of the precision when its estimate is lower
+// (16 rows on the mixed path for large grids, whose halo rows are fewer: 1947 against 2125 us per
+// launch at 256^3; 4 rows on the FP64 path for grids with too few tiles).
+int default_rows(const Grid& g) {
+  const Grid* one[1] = {&g};
+  double e8, eo;
+  const int other = g.prec == M2C_MIXED ? 16 : 4;
+  choose_tz(one, 1, tile_shape(g.prec, 8), &e8);
+  choose_tz(one, 1, tile_shape(g.prec, other), &eo);
+  return eo < e8 ? other : 8;
 }
 
 // Event pairs recorded around launches while profiling, tagged with the kernel kind.
@@ -1301,11 +1355,16 @@ m2c_status m2c_batch_create(m2c_batch** out, m2c_ctx** v, int k, void* workspace
                                                      align_up(sizeof(long long) * (size_t)(k + 1)));
   b->tiles.assign(k + 1, 0);
   b->nmax = 1;
+  if (tz <= 0) {
+    std::vector<const Grid*> gs;
+    for (int i = 0; i < k; ++i) gs.push_back(&v[i]->host);
+    tz = choose_tz(gs.data(), k, tile_shape(v[0]->host.prec, ty));
+  }
   for (int i = 0; i < k; ++i) {
     m2c_ctx* c = v[order[i]];
     b->ctx.push_back(c);
     Grid g = c->host;
-    set_tiling(g, ty, tz > 0 ? tz : default_tz(g, ty));
+    set_tiling(g, ty, tz);
     b->hosts.push_back(g);
     b->tiles[i + 1] = b->tiles[i] + ntiles_of(g);
     b->nmax = std::max(b->nmax, g.N);
