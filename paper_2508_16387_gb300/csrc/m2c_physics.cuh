@@ -30,6 +30,8 @@ struct EosP {
   R g, pc, gm1, gpc, inv_gm1;                // SG and NASG
   R rho0, c0, s, G0, e0, eta_min;            // MG
   R K0, rg, inv_rg, inv_2rho0, eta_max, pmin, rk4_span;  // MG derived
+  R gm, ex, two_gm1, inv_g;                  // SG: (g-1)/(g+1), (g-1)/(2g), 2/(g-1), 1/g (Riemann wave curves)
+  R rmax, sG, gk, kap, kap2;                 // MG: rho0 s/(s-1), s - G0, G0/K0, (K0 rho0)^-1/2, 1/(K0 rho0)
   R b, ec;                                   // NASG
   R om, A1, A2, R1r, R2r, c1, c2;            // JWL: w, A_i, R_i rho0, w/(R_i rho0)
 };
@@ -46,6 +48,10 @@ __host__ inline EosP<R> make_eos(int type, const double* prm) {
     e.gm1 = (R)(prm[0] - 1.0);
     e.gpc = (R)(prm[0] * prm[1]);
     e.inv_gm1 = (R)(1.0 / (prm[0] - 1.0));
+    e.gm = (R)((prm[0] - 1.0) / (prm[0] + 1.0));
+    e.ex = (R)((prm[0] - 1.0) / (2.0 * prm[0]));
+    e.two_gm1 = (R)(2.0 / (prm[0] - 1.0));
+    e.inv_g = (R)(1.0 / prm[0]);
   } else if (type == M2C_EOS_NASG) {
     e.g = (R)prm[0];
     e.pc = (R)prm[1];
@@ -78,22 +84,28 @@ __host__ inline EosP<R> make_eos(int type, const double* prm) {
     e.eta_max = (R)(1.0 / prm[2]);
     e.pmin = (R)(K0 * prm[5]);
     e.rk4_span = (R)(0.05 * K0);
+    e.rmax = (R)(prm[0] * prm[2] / (prm[2] - 1.0));
+    e.sG = (R)(prm[2] - prm[3]);
+    e.gk = (R)(prm[3] / K0);
+    e.kap2 = (R)(1.0 / (K0 * prm[0]));
+    e.kap = (R)sqrt(1.0 / (K0 * prm[0]));
   }
   return e;
 }
 
 __host__ inline EosDev make_eos_dev(int type, const double* prm) { return make_eos<double>(type, prm); }
 
-// Division, reciprocal and square root of the working precision. FP64: the
-// quotient and reciprocal of div_nr / rcp_nr below (a binary32 seed refined by
-// Newton-Raphson steps; the quotient takes a residual correction and equals the
-// IEEE quotient, the reciprocal is within an ulp), IEEE square root. FP32 half
+// Division, reciprocal and square root of the working precision. FP64: those of
+// div_nr, rcp_nr and sqrt_nr below (a corrected binary32 seed; the quotient takes
+// a residual correction and equals the IEEE quotient, the reciprocal and the
+// root are within an ulp). FP32 half
 // of the mixed path: the hardware approximations (a few ulp), far below the
 // FP32 rounding already accepted there.
 __device__ __forceinline__ double rcp_nr(double b);
 __device__ __forceinline__ double div_nr(double a, double b);
 __device__ __forceinline__ bool nr_range(double b);
 __device__ __forceinline__ double rcp_nr_in_range(double b);
+__device__ __forceinline__ double sqrt_nr(double x);
 template <typename R>
 __device__ __forceinline__ R rdiv(R a, R b) {
   if constexpr (sizeof(R) == 8) return div_nr(a, b);
@@ -106,7 +118,7 @@ __device__ __forceinline__ R rrcp(R x) {
 }
 template <typename R>
 __device__ __forceinline__ R rsqrt_pos(R x) {  // sqrt of x > 0
-  if constexpr (sizeof(R) == 8) return sqrt(x);
+  if constexpr (sizeof(R) == 8) return sqrt_nr(x);
   else return x * rsqrtf(x);
 }
 
@@ -299,50 +311,65 @@ __host__ __device__ __forceinline__ void d2f_group(const double (&x)[K], float (
 #endif
 }
 
-// FP64 reciprocal and quotient for the bulk kernels: a binary32 seed of 1/b
-// (b's leading 23 mantissa bits, then the hardware's approximate binary32
-// reciprocal; relative error below 2^-21 together), refined by two
-// Newton-Raphson steps x <- x + x (1 - b x), each of which squares the
-// relative error, to 1/b within an ulp; the quotient a x then takes one
+// FP64 reciprocal, quotient and roots: a binary32 seed from b's leading 23
+// mantissa bits (the hardware's approximate binary32 function; relative error
+// below 2^-21 together), corrected by one third-order step, whose truncation is
+// below 2^-62: 1/b = x (1 + e + e^2 + ...) with e = 1 - b x, and 1/sqrt(b) =
+// y (1 + e/2 + 3 e^2/8 + ...) with e = 1 - b y^2. The seed stays on the integer
+// and special-function pipes; an FP64 instruction occupies its scheduler's FP64
+// unit for 64 cycles (measured, whatever the number of active lanes), so
+// the count of them is the cost: 3 for the reciprocal (4 with two
+// Newton-Raphson steps), 5 for a root (8). The quotient q = a x takes one
 // residual correction q <- q + (a - b q) x (Markstein, IBM J. Res. Dev. 34,
-// 1990). The seed stays on the integer and special-function pipes. For |b|
-// outside [2^-125, 2^125) (zeros, infinities, NaNs included) the IEEE
-// operations. Both are checked against IEEE 1/b and a/b on the device.
+// 1990). For |b| outside [2^-125, 2^125) (zeros, infinities, NaNs included) the
+// IEEE operations, out of line so that the call sites stay short. All are checked
+// against the IEEE operations on the device.
 __device__ __forceinline__ bool nr_range(double b) {
   return (hi_of(b) & 0x7fffffffu) - 0x38200000u < 0x47c00000u - 0x38200000u;
 }
+// the same for b > 0 (false for negative b)
+__device__ __forceinline__ bool nr_range_pos(double b) { return hi_of(b) - 0x38200000u < 0x47c00000u - 0x38200000u; }
+static __device__ __noinline__ double rcp_ieee(double b) { return 1.0 / b; }
+static __device__ __noinline__ double div_ieee(double a, double b) { return a / b; }
+static __device__ __noinline__ double sqrt_ieee(double x) { return sqrt(x); }
 __device__ __forceinline__ double rcp_nr_in_range(double b) {
   const unsigned hi = hi_of(b), ah = hi & 0x7fffffffu;
   const float f = float_of((((ah - 0x38000000u) << 3) | (lo_of(b) >> 29)) | (hi & 0x80000000u));
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
   const unsigned rb = bits_of(r), ra = rb & 0x7fffffffu;
-  double x = double_of_words(((ra >> 3) + (896u << 20)) | (rb & 0x80000000u), ra << 29);
-  x = fma(x, fma(-b, x, 1.0), x);
-  x = fma(x, fma(-b, x, 1.0), x);
-  return x;
+  const double x = double_of_words(((ra >> 3) + (896u << 20)) | (rb & 0x80000000u), ra << 29);
+  const double e = fma(-b, x, 1.0);
+  return fma(x, fma(e, e, e), x);
 }
 __device__ __forceinline__ double rcp_nr(double b) {
   if (nr_range(b)) return rcp_nr_in_range(b);
-  return 1.0 / b;
+  return rcp_ieee(b);
 }
-// FP64 reciprocal square root 1/sqrt(x), x > 0, for the Mie-Grueneisen
-// isentrope integrand: a binary32 seed (x's leading 23 mantissa bits, then the
-// hardware's approximate binary32 reciprocal square root, relative error below
-// 2^-21), refined by two Newton-Raphson steps y <- y + y (1 - x y^2)/2 in FP64
-// (each squares the relative error up to a factor 3/2), within an ulp or two of
-// 1/sqrt(x); x outside [2^-125, 2^125) takes 1/sqrt(x) with the IEEE operations.
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  if (!nr_range(x)) return 1.0 / sqrt(x);
-  const unsigned hi = hi_of(x);
-  const float f = float_of(((hi - 0x38000000u) << 3) | (lo_of(x) >> 29));
+// binary32 seed of 1/sqrt(x), x > 0 in the Newton range
+__device__ __forceinline__ double rsqrt_seed(double x) {
+  const float f = float_of(((hi_of(x) - 0x38000000u) << 3) | (lo_of(x) >> 29));
   float r;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
   const unsigned rb = bits_of(r);
-  double y = double_of_words((rb >> 3) + (896u << 20), rb << 29);
-  y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
-  y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
-  return y;
+  return double_of_words((rb >> 3) + (896u << 20), rb << 29);
+}
+// 1/sqrt(x), x > 0, within two ulps
+__device__ __forceinline__ double rsqrt_nr_in_range(double x) {
+  const double y = rsqrt_seed(x);
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double rsqrt_nr(double x) {
+  if (!nr_range_pos(x)) return rcp_ieee(sqrt_ieee(x));
+  return rsqrt_nr_in_range(x);
+}
+// sqrt(x), x >= 0, within an ulp: the same correction applied to x y
+__device__ __forceinline__ double sqrt_nr(double x) {
+  if (!nr_range_pos(x)) return sqrt_ieee(x);
+  const double y = rsqrt_seed(x), t = x * y;
+  const double e = fma(-t, y, 1.0);
+  return fma(t * e, fma(0.375, e, 0.5), t);
 }
 
 // The corrected quotient is the IEEE one when it is a normal number and its
@@ -357,7 +384,7 @@ __device__ __forceinline__ double div_nr(double a, double b) {
     if (ea - 126u < 1795u) return fma(fma(-b, q, a), x, q);
     if (((ha & 0x7fffffffu) | lo_of(a)) == 0u) return q;
   }
-  return a / b;
+  return div_ieee(a, b);
 }
 
 template <typename R>
@@ -496,11 +523,11 @@ __device__ __forceinline__ R va_slope(R a, R b) {
   R ab = a * b;
   if constexpr (sizeof(R) == 8) {
     // FP64: the sign test on the bits and the quotient as the product with the
-    // Newton-Raphson reciprocal (within an ulp or two of the IEEE quotient, which
-    // is taken where the denominator is outside the reciprocal's range)
+    // corrected reciprocal (within an ulp or two of the IEEE quotient, which is
+    // taken where the denominator is outside the reciprocal's range)
     if (!gt0(ab)) return 0.0;
     const double num = ab * (a + b), den = a * a + b * b;
-    return nr_range(den) ? num * rcp_nr_in_range(den) : num / den;
+    return nr_range(den) ? num * rcp_nr_in_range(den) : div_ieee(num, den);
   } else {
     if (!(ab > (R)0)) return (R)0;
     return rdiv<R>(ab * (a + b), a * a + b * b);

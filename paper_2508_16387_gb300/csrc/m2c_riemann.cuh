@@ -23,31 +23,49 @@ constexpr double kHugTol = 1e-14;
 constexpr int kHugCap = 100;
 constexpr int kRk4Steps = 64;
 
+// One side of a problem with what its wave curve needs at every pressure.
 struct Side {
   double rho, u, p, c, e;
+  // SG: p + p_c, its reciprocal, rho c, 2 c/(g - 1), and the shock constants 2/((g + 1) rho),
+  // (g - 1)/(g + 1) (p + p_c)
+  double pb, ipb, z, cf, A, B;
+  // MG: 1/rho, 1/c^2; last Hugoniot root and its slope at pressure hp (NaN: none)
+  double iv, ic2, hp, hr, hd;
   int nrk;  // RK4 substeps of this side's MG rarefaction curve in one problem; 0: per evaluation
   // MG: spacing of the problem's fixed RK4 nodes p_K - i dnode (0: none), and the
   // isentrope state (rho, f) after the first mbase full substeps, kept between the
   // evaluations of one problem (nearby pressures share their nodes)
   int mbase;
-  double dnode, dspan, rbase, fbase;  // dspan = nrk dnode, the span bound the nodes cover
+  double dnode, idnode, dspan, rbase, fbase;  // dspan = nrk dnode, the span bound the nodes cover
 };
 
 __device__ inline bool make_side(const EosDev& q, double rho, double u, double p, Side& K) {
-  if (!(rho > 0.0)) return false;
-  double e, c2;
-  if (!eos_e_c2<double, true>(q, rho, 1.0 / rho, p, e, c2)) return false;
+  double e = 0.0, c2 = 0.0;
+  const double iv = rcp_nr(rho);
+  if (!eos_e_c2<double, true>(q, rho, iv, p, e, c2)) return false;
   K.rho = rho;
   K.u = u;
   K.p = p;
-  K.c = sqrt(c2);
+  K.c = sqrt_nr(c2);
   K.e = e;
-  K.nrk = 0;
-  K.mbase = 0;
-  K.dnode = 0.0;
-  K.dspan = 0.0;
-  K.rbase = rho;
-  K.fbase = 0.0;
+  if (q.type == M2C_EOS_SG) {
+    K.pb = p + q.pc;
+    K.ipb = rcp_nr(K.pb);
+    K.z = rho * K.c;
+    K.cf = q.two_gm1 * K.c;
+    K.A = (1.0 - q.gm) * iv;
+    K.B = q.gm * K.pb;
+  } else {
+    K.iv = iv;
+    K.ic2 = rcp_nr(c2);
+    K.hp = NAN;
+    K.nrk = 0;
+    K.mbase = 0;
+    K.dnode = 0.0;
+    K.dspan = 0.0;
+    K.rbase = rho;
+    K.fbase = 0.0;
+  }
   return true;
 }
 
@@ -62,7 +80,7 @@ __device__ inline double eos_plow(const EosDev& q) {
 // Equal RK4 substeps over a pressure span dp of an MG isentrope: 64 for a span
 // of at least 5% of K0 = rho0 c0^2, proportionally fewer (at least one) below.
 __device__ inline int mg_substeps(const EosDev& q, double dp) {
-  double nsd = ceil(__ddiv_rn(kRk4Steps * fabs(dp), q.rk4_span));
+  double nsd = ceil(div_nr(kRk4Steps * fabs(dp), q.rk4_span));  // div_nr: the IEEE quotient
   nsd = nsd >= 1.0 ? (nsd > kRk4Steps ? (double)kRk4Steps : nsd) : 1.0;
   return (int)nsd;
 }
@@ -88,13 +106,14 @@ __device__ inline void fix_substeps(const EosDev& qL, Side& L, const EosDev& qR,
   const double ZL = __dmul_rn(L.rho, L.c), ZR = __dmul_rn(Rs.rho, Rs.c);
   const double num = __dsub_rn(__dadd_rn(__dmul_rn(ZR, L.p), __dmul_rn(ZL, Rs.p)),
                                __dmul_rn(__dmul_rn(ZL, ZR), __dsub_rn(Rs.u, L.u)));
-  const double pac = __ddiv_rn(num, __dadd_rn(ZL, ZR));
+  const double pac = div_nr(num, __dadd_rn(ZL, ZR));
   const double loL = fmax(plow, fmin(Rs.p, pac)), loR = fmax(plow, fmin(L.p, pac));
   // MG: the count for the span bound and the spacing of the fixed nodes (span / count)
   auto mg_nodes = [](const EosDev& q, Side& K, double lo) {
     const double span = fmax(__dsub_rn(K.p, lo), 0.0);
     K.nrk = mg_substeps(q, span);
-    K.dnode = (span > 0.0 && isfinite(span)) ? __ddiv_rn(span, (double)K.nrk) : 0.0;
+    K.dnode = (span > 0.0 && isfinite(span)) ? div_nr(span, (double)K.nrk) : 0.0;
+    K.idnode = rcp_nr(K.dnode);
     K.dspan = __dmul_rn((double)K.nrk, K.dnode);
   };
   if (qL.type == M2C_EOS_MG) mg_nodes(qL, L, loL);
@@ -103,101 +122,110 @@ __device__ inline void fix_substeps(const EosDev& qL, Side& L, const EosDev& qR,
   if (qR.type == M2C_EOS_JWL) Rs.nrk = jwl_substeps(Rs.p, loR);
 }
 
-__device__ inline int wave_sg(const EosDev& q, const Side& K, double p, double& f, double& df, double& rs,
-                              bool want_rho = true, double* drs = nullptr) {
-  const double g = q.g, pb = p + q.pc, pbK = K.p + q.pc;
-  if (!(pb >= 0.0) || !(pbK > 0.0)) return M2C_ENONPHYS;
+// One side's wave curve at a pressure: f and f', and what the star density
+// behind the wave follows from (a: SG rarefaction the power r^((g-1)/(2g)), MG
+// shock and rarefaction rho*; b: MG d rho*/dp; NASG and JWL rho* and its slope).
+struct Wave {
+  double f, df, a, b;
+};
+
+// The solver's control flow has one entry and one exit per block (flags instead
+// of returns inside loops), so that the lanes of a warp meet again after every
+// branch and loop: with returns inside the loops a warp executed 12-15 Newton
+// iterations and 90-140 isentrope substeps for an average of 3 and 30 a face
+// (late shock-bubble), the lanes taking turns.
+__device__ inline int wave_sg(const EosDev& q, const Side& K, double p, Wave& w) {
+  const double pb = p + q.pc, dp = p - K.p;
   if (p > K.p) {
-    double A = 2.0 / ((g + 1.0) * K.rho);
-    double B = (g - 1.0) / (g + 1.0) * pbK;
-    double sq = sqrt(A / (pb + B));
-    f = (p - K.p) * sq;
-    df = sq * (1.0 - 0.5 * (p - K.p) / (pb + B));
-    double r = pb / pbK, gm = (g - 1.0) / (g + 1.0);
-    rs = K.rho * (r + gm) / (gm * r + 1.0);
-    if (drs) *drs = K.rho * (1.0 - gm * gm) / ((gm * r + 1.0) * (gm * r + 1.0) * pbK);
+    // f = dp sqrt(A/(pb + B)), f' = sqrt(A/(pb + B)) (1 - dp/(2 (pb + B)))
+    const double iD = rcp_nr(pb + K.B), sq = sqrt_nr(K.A * iD);
+    w.f = dp * sq;
+    w.df = sq * fma(-0.5 * dp, iD, 1.0);
   } else {
-    // one power serves f and f': r^{-(g+1)/(2g)} = r^{(g-1)/(2g)} / r; the density
-    // behind the wave is only evaluated when asked for (after the iteration)
-    const double r = pb / pbK;
-    const double q = pow(r, (g - 1.0) / (2.0 * g));
-    f = 2.0 * K.c / (g - 1.0) * (q - 1.0);
-    df = q / (r * K.rho * K.c);
-    rs = want_rho ? K.rho * pow(r, 1.0 / g) : 0.0;
-    if (drs) *drs = rs / (g * pb);
+    // one power serves f, f' (r^{-(g+1)/(2g)} = r^{(g-1)/(2g)} / r) and, after
+    // the iteration, the density; r is the IEEE quotient (exactly 1 at p = p_K)
+    const double r0 = pb * K.ipb, r = fma(fma(-K.pb, r0, pb), K.ipb, r0);
+    const double pw = pow(r, q.ex);
+    w.f = K.cf * (pw - 1.0);
+    w.df = pw * rcp_nr(r * K.z);
+    w.a = pw;
   }
-  return M2C_OK;
+  return pb >= 0.0 && K.pb > 0.0 ? M2C_OK : M2C_ENONPHYS;
 }
 
-// de/drho at constant p for MG
-__device__ inline bool mg_dedr(const EosDev& q, double rho, double& dedr) {
-  double eta = 1.0 - div_nr(q.rho0, rho);
-  if (!(eta < q.eta_max)) return false;
-  double pR, dpR, eR, deR;
-  mg_ref<double>(q, eta, pR, dpR, eR, deR);
-  dedr = div_nr((deR - dpR * q.inv_rg) * q.rho0, rho * rho);
-  return true;
-}
-
-// Density on the MG Hugoniot through K at pressure p (safeguarded Newton in a
-// closed bracket, stopped at the first step below the tolerance) and d rho/dp
-// along it.
-__device__ inline int mg_hugoniot(const EosDev& q, const Side& K, double p, double& rho_out, double& drdp) {
-  double lo = K.rho, hi = q.rho0 * q.s / (q.s - 1.0);
-  if (!(hi > lo)) return M2C_ENONPHYS;
-  double rho = K.rho + div_nr(p - K.p, K.c * K.c);
+// Density on the MG Hugoniot through K at pressure p > p_K (safeguarded Newton
+// in a closed bracket, stopped at the first step below the tolerance) and
+// d rho/dp along it. The start is the root of the problem's previous evaluation
+// moved along its slope, else the acoustic density.
+__device__ inline int mg_hugoniot(const EosDev& q, Side& K, double p, double& rho_out, double& drdp) {
+  double lo = K.rho, hi = q.rmax;
+  bool more = hi > lo;
+  int st = more ? M2C_OK : M2C_ENONPHYS;
+  double rho = K.hp == K.hp ? fma(K.hd, p - K.hp, K.hr) : fma(p - K.p, K.ic2, K.rho);
   if (!(rho > lo && rho < hi)) rho = 0.5 * (lo + hi);
-  bool done = false;
-  for (int it = 0; it < kHugCap; ++it) {
-    double eta = 1.0 - div_nr(q.rho0, rho);
-    if (!(eta < q.eta_max)) return M2C_ENONPHYS;
-    double pR, dpR, eR, deR;
+  const double hp = 0.5 * (p + K.p);
+  double dH = 1.0;
+  for (int it = 0; more; ++it) {
+    const double iv = rcp_nr(rho), eta = fma(-q.rho0, iv, 1.0);
+    double pR = 0.0, dpR = 0.0, eR = 0.0, deR = 0.0;
     mg_ref<double>(q, eta, pR, dpR, eR, deR);
-    double e = eR + (p - pR) * q.inv_rg;
-    double dedr = div_nr((deR - dpR * q.inv_rg) * q.rho0, rho * rho);
-    double H = e - K.e - 0.5 * (p + K.p) * (div_nr(1.0, K.rho) - div_nr(1.0, rho));
-    double dH = dedr - div_nr(0.5 * (p + K.p), rho * rho);
+    const double H = fma(p - pR, q.inv_rg, eR) - K.e - hp * (K.iv - iv);
+    dH = fma(fma(-dpR, q.inv_rg, deR), q.rho0, -hp) * (iv * iv);
     if (H > 0.0) lo = rho; else hi = rho;
-    double rn = rho - div_nr(H, dH);
+    double rn = fma(-H, rcp_nr(dH), rho);
     if (!(rn >= lo && rn <= hi)) rn = 0.5 * (lo + hi);
-    bool conv = fabs(rn - rho) <= kHugTol * rn;
+    const bool conv = fabs(rn - rho) <= kHugTol * rn;
     rho = rn;
-    if (conv) { done = true; break; }
+    if (!(eta < q.eta_max)) st = M2C_ENONPHYS;
+    else if (!conv && it + 1 == kHugCap) st = M2C_ENOCONV;
+    more = st == M2C_OK && !conv;
   }
-  if (!done) return M2C_ENOCONV;
-  double dedr;
-  if (!mg_dedr(q, rho, dedr)) return M2C_ENONPHYS;
-  double Hp = q.inv_rg - 0.5 * (div_nr(1.0, K.rho) - div_nr(1.0, rho));
-  double Hr = dedr - div_nr(0.5 * (p + K.p), rho * rho);
+  // along the Hugoniot d rho/dp = -H_p/H_rho, the slope H_rho from the last iterate
+  const double Hp = q.inv_rg - 0.5 * (K.iv - rcp_nr(rho));
   rho_out = rho;
-  drdp = -div_nr(Hp, Hr);
-  return M2C_OK;
+  drdp = -Hp * rcp_nr(dH);
+  K.hp = p;
+  K.hr = rho;
+  K.hd = drdp;
+  return st;
 }
 
-// d rho/dp = 1/c^2 and df/dp = 1/(rho c) of the isentrope from one reciprocal
-// square root of c^2 and the reciprocal of rho (each within an ulp or two of the
-// correctly rounded value).
-__device__ inline int mg_rhs(const EosDev& q, double p, double rho, double& drho, double& dfv) {
-  double e, c2;
-  const double ir = rcp_nr(rho);
-  if (!eos_e_c2<double>(q, rho, ir, p, e, c2)) return M2C_ENONPHYS;
-  const double y = rsqrt_nr(c2);
-  drho = y * y;
-  dfv = y * ir;
-  return M2C_OK;
+// Right-hand side of the MG isentrope. With d = rho - rho0 and q = rho - s d
+// (1 - s eta = q/rho), the sound speed of the compression branch is
+//   rho^2 c^2 = K0 rho0 A,  A = (rho + (s - G0) d) rho^2/q^3 + (G0/K0) p,
+// and that of the tension branch A = (rho - G0 d)/rho + (G0/K0) p (s = 0, the
+// factor 1/rho instead of rho^2/q^3). So d rho/dp = 1/c^2 = (rho y)^2/(K0 rho0)
+// and df/dp = 1/(rho c) = y/(K0 rho0)^(1/2) with y = A^(-1/2): 17 FP64
+// instructions with one reciprocal and one root (35 through the general e and
+// c^2); the constant factors sit in the substep lengths. gp = (G0/K0) p. ok is
+// cleared outside the EOS domain (rho <= 0, eta >= 1/s, c^2 <= 0). A finite
+// tension cutoff takes the general sound speed.
+__device__ inline void mg_rhs(const EosDev& q, double gp, double rho, double& kr, double& y, bool& ok) {
+  const double d = rho - q.rho0;
+  const bool comp = gt0(d);
+  const double qq = fma(comp ? -q.s : 0.0, d, rho), n = fma(comp ? q.sG : -q.G0, d, rho);
+  ok = ok && gt0(rho) && nr_range_pos(qq);
+  const double iq = rcp_nr_in_range(qq);
+  const double t = comp ? rho * iq : 1.0;
+  double A = fma(n, t * t * iq, gp);
+  if (q.eta_min > -INFINITY && q.rho0 * rcp_nr(rho) > 1.0 - q.eta_min) A = gp - q.gk * q.pmin;
+  ok = ok && nr_range_pos(A);
+  y = rsqrt_nr_in_range(A);
+  const double ry = rho * y;
+  kr = ry * ry;
 }
 
 // One classical RK4 substep of the MG isentrope (rho, f) from pressure pi by hs.
-__device__ inline int mg_rk4_substep(const EosDev& q, double pi, double hs, double& rho, double& fv) {
-  double k1r, k1f, k2r, k2f, k3r, k3f, k4r, k4f;
-  int st = mg_rhs(q, pi, rho, k1r, k1f);
-  if (!st) st = mg_rhs(q, pi + 0.5 * hs, rho + 0.5 * hs * k1r, k2r, k2f);
-  if (!st) st = mg_rhs(q, pi + 0.5 * hs, rho + 0.5 * hs * k2r, k3r, k3f);
-  if (!st) st = mg_rhs(q, pi + hs, rho + hs * k3r, k4r, k4f);
-  if (st) return st;
-  rho = rho + hs / 6.0 * (k1r + 2.0 * k2r + 2.0 * k3r + k4r);
-  fv = fv + hs / 6.0 * (k1f + 2.0 * k2f + 2.0 * k3f + k4f);
-  return M2C_OK;
+__device__ inline void mg_rk4_substep(const EosDev& q, double pi, double hs, double& rho, double& fv, bool& ok) {
+  const double g0 = q.gk * pi, gh = q.gk * hs, gm = fma(0.5, gh, g0);
+  const double hr = hs * q.kap2, h2 = 0.5 * hr;
+  double k1, k2, k3, k4, y1, y2, y3, y4;
+  mg_rhs(q, g0, rho, k1, y1, ok);
+  mg_rhs(q, gm, fma(h2, k1, rho), k2, y2, ok);
+  mg_rhs(q, gm, fma(h2, k2, rho), k3, y3, ok);
+  mg_rhs(q, g0 + gh, fma(hr, k3, rho), k4, y4, ok);
+  rho = fma(hr * (1.0 / 6.0), fma(2.0, k2 + k3, k1 + k4), rho);
+  fv = fma(hs * (q.kap * (1.0 / 6.0)), fma(2.0, y2 + y3, y1 + y4), fv);
 }
 
 // MG wave curve. Rarefaction: the isentrope integrated by classical RK4 in p;
@@ -205,72 +233,70 @@ __device__ inline int mg_rk4_substep(const EosDev& q, double pi, double hs, doub
 // down to the last node above p, resumed from the node reached by an earlier
 // evaluation of the problem when it lies at or below, then one partial substep
 // to p): the curve is continuous and smooth in p; beyond the bound, and for a
-// wave evaluated alone, equal substeps over p_K - p. The node arithmetic is
+// wave evaluated alone, equal substeps over p_K - p. Both are one loop, so that
+// the lanes of a warp take their substeps together. The node arithmetic is
 // written without contracted multiply-adds, so that it takes the same nodes as
 // the oracle.
-__device__ inline int wave_mg(const EosDev& q, Side& K, double p, double& f, double& df, double& rs,
-                              double* drs = nullptr) {
+__device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
+  int st = M2C_OK;
   if (p == K.p) {
-    f = 0.0;
-    df = 1.0 / (K.rho * K.c);
-    rs = K.rho;
-    if (drs) *drs = 1.0 / (K.c * K.c);
-    return M2C_OK;
-  }
-  if (p > K.p) {
+    w.f = 0.0;
+    w.df = K.iv * rcp_nr(K.c);
+    w.a = K.rho;
+    w.b = K.ic2;
+  } else if (p > K.p) {
     double rho, drdp;
-    int st = mg_hugoniot(q, K, p, rho, drdp);
-    if (st) return st;
-    double dv = div_nr(1.0, K.rho) - div_nr(1.0, rho);
-    double fv = sqrt((p - K.p) * dv);
-    f = fv;
-    df = div_nr(dv + div_nr((p - K.p) * drdp, rho * rho), 2.0 * fv);
-    rs = rho;
-    if (drs) *drs = drdp;
-    return M2C_OK;
-  }
-  double rho = K.rho, fv = 0.0;
-  const double dp = __dsub_rn(K.p, p);
-  // (one node interval: the partial substep from p_K is the single equal substep
-  // over p_K - p, the same arithmetic, so that case takes the short path)
-  if (K.nrk > 1 && K.dnode > 0.0 && dp < K.dspan) {
-    int m = (int)floor(div_nr(dp, K.dnode));  // div_nr: the IEEE quotient
-    if (m > K.nrk - 1) m = K.nrk - 1;
-    if (K.mbase > m) {  // an earlier evaluation went past this node: start over from p_K
-      K.mbase = 0;
-      K.rbase = K.rho;
-      K.fbase = 0.0;
-    }
-    rho = K.rbase;
-    fv = K.fbase;
-    for (int i = K.mbase; i < m; ++i) {
-      const int st = mg_rk4_substep(q, __dsub_rn(K.p, __dmul_rn((double)i, K.dnode)), -K.dnode, rho, fv);
-      if (st) return st;
-    }
-    K.mbase = m;
-    K.rbase = rho;
-    K.fbase = fv;
-    const double hp = __dsub_rn(dp, __dmul_rn((double)m, K.dnode));
-    if (hp > 0.0) {
-      const int st = mg_rk4_substep(q, __dsub_rn(K.p, __dmul_rn((double)m, K.dnode)), -hp, rho, fv);
-      if (st) return st;
-    }
+    st = mg_hugoniot(q, K, p, rho, drdp);
+    const double ir = rcp_nr(rho), dv = K.iv - ir, dp = p - K.p;
+    const double fv = sqrt_nr(dp * dv);
+    w.f = fv;
+    w.df = fma(dp * drdp, ir * ir, dv) * rcp_nr(2.0 * fv);
+    w.a = rho;
+    w.b = drdp;
   } else {
-    // equal substeps: the problem's count (beyond its span bound), else chosen for this span
-    const int ns = K.nrk > 0 ? K.nrk : mg_substeps(q, p - K.p);
-    const double hs = (p - K.p) / ns;
-    for (int i = 0; i < ns; ++i) {
-      const int st = mg_rk4_substep(q, K.p + i * hs, hs, rho, fv);
-      if (st) return st;
+    const double dp = __dsub_rn(K.p, p);
+    const bool within = K.nrk > 1 && K.dnode > 0.0 && dp < K.dspan;
+    double rho = K.rho, fv = 0.0, gap = 0.0, last = dp;
+    int i = 0, m = 0;
+    if (within) {
+      const double m0 = dp * K.idnode;
+      m = (int)floor(fma(fma(-K.dnode, m0, dp), K.idnode, m0));  // the IEEE quotient dp/dnode
+      if (m > K.nrk - 1) m = K.nrk - 1;
+      if (K.mbase <= m) {  // resume from the deepest node, unless an earlier evaluation went past m
+        i = K.mbase;
+        rho = K.rbase;
+        fv = K.fbase;
+      }
+      gap = K.dnode;
+    } else {
+      // the problem's count (beyond its span bound), else one chosen for this span; a
+      // count of one is a single substep, the partial one below
+      const int ns = K.nrk > 0 ? K.nrk : mg_substeps(q, dp);
+      if (ns > 1) {
+        m = ns;
+        gap = div_nr(dp, (double)ns);
+        last = 0.0;
+      }
     }
+    bool ok = true;
+    for (; i < m; ++i) mg_rk4_substep(q, __dsub_rn(K.p, __dmul_rn((double)i, gap)), -gap, rho, fv, ok);
+    const double pm = __dmul_rn((double)m, gap);
+    if (within) {
+      K.mbase = m;
+      K.rbase = rho;
+      K.fbase = fv;
+      last = __dsub_rn(dp, pm);
+    }
+    if (last > 0.0) mg_rk4_substep(q, __dsub_rn(K.p, pm), -last, rho, fv, ok);
+    double k, y;
+    mg_rhs(q, q.gk * p, rho, k, y, ok);
+    w.f = fv;
+    w.df = y * q.kap;
+    w.a = rho;
+    w.b = k * q.kap2;
+    if (!ok) st = M2C_ENONPHYS;
   }
-  double e, c2;
-  if (!eos_e_c2<double>(q, rho, 1.0 / rho, p, e, c2)) return M2C_ENONPHYS;
-  f = fv;
-  df = 1.0 / (rho * sqrt(c2));
-  rs = rho;
-  if (drs) *drs = 1.0 / c2;
-  return M2C_OK;
+  return st;
 }
 
 // NASG wave curves in P = p + p_c and the covolume-reduced specific volume
@@ -279,8 +305,8 @@ __device__ inline int wave_mg(const EosDev& q, Side& K, double p, double& f, dou
 // f = (p - p_K) sqrt(A/(P + gm P_K)) with A = 2 w_K/(g + 1). Rarefaction: the
 // isentrope P w^g = const gives rho c = sqrt(g P / w) and
 // f = 2 c_K (1 - b rho_K)/(g - 1) (r^((g-1)/(2g)) - 1).
-static __device__ __noinline__ int wave_nasg(const EosDev& q, const Side& K, double p, double& f, double& df,
-                                             double& rs, double* drs) {
+static __device__ __noinline__ int wave_nasg(const EosDev& q, const Side& K, double p, Wave& wv) {
+  double &f = wv.f, &df = wv.df, &rs = wv.a, &drs = wv.b;
   const double g = q.g, b = q.b, P = p + q.pc, PK = K.p + q.pc, wK = 1.0 / K.rho - b;
   if (!(P >= 0.0) || !(PK > 0.0) || !(wK > 0.0)) return M2C_ENONPHYS;
   const double r = P / PK;
@@ -291,13 +317,13 @@ static __device__ __noinline__ int wave_nasg(const EosDev& q, const Side& K, dou
     df = sq * (1.0 - 0.5 * (p - K.p) / D);
     const double w = wK * (gm * r + 1.0) / (r + gm);
     rs = 1.0 / (b + w);
-    if (drs) *drs = rs * rs * wK * (1.0 - gm * gm) / ((r + gm) * (r + gm) * PK);
+    drs = rs * rs * wK * (1.0 - gm * gm) / ((r + gm) * (r + gm) * PK);
   } else {
     f = 2.0 * K.c * (1.0 - b * K.rho) / (g - 1.0) * (pow(r, (g - 1.0) / (2.0 * g)) - 1.0);
     const double w = wK * pow(r, -1.0 / g);
     df = sqrt(w / (g * P));
     rs = 1.0 / (b + w);
-    if (drs) *drs = rs * rs * w / (g * P);
+    drs = rs * rs * w / (g * P);
   }
   return M2C_OK;
 }
@@ -351,13 +377,13 @@ __device__ inline int jwl_hugoniot(const EosDev& q, const Side& K, double p, dou
 // the isentrope d rho/dp = 1/c^2, df/dp = 1/(rho c) integrated by classical RK4
 // in s = ln p on equal substeps (fixed per problem, fix_substeps; else for
 // this span); it needs p > 0.
-static __device__ __noinline__ int wave_jwl(const EosDev& q, const Side& K, double p, double& f, double& df,
-                                            double& rs, double* drs) {
+static __device__ __noinline__ int wave_jwl(const EosDev& q, const Side& K, double p, Wave& wv) {
+  double &f = wv.f, &df = wv.df, &rs = wv.a, &drs = wv.b;
   if (p == K.p) {
     f = 0.0;
     df = 1.0 / (K.rho * K.c);
     rs = K.rho;
-    if (drs) *drs = 1.0 / (K.c * K.c);
+    drs = 1.0 / (K.c * K.c);
     return M2C_OK;
   }
   if (p > K.p) {
@@ -369,7 +395,7 @@ static __device__ __noinline__ int wave_jwl(const EosDev& q, const Side& K, doub
     f = fv;
     df = (dv + (p - K.p) * drdp / (rho * rho)) / (2.0 * fv);
     rs = rho;
-    if (drs) *drs = drdp;
+    drs = drdp;
     return M2C_OK;
   }
   if (!(p > 0.0) || !(K.p > 0.0)) return M2C_ENONPHYS;
@@ -404,40 +430,101 @@ static __device__ __noinline__ int wave_jwl(const EosDev& q, const Side& K, doub
   f = fv;
   df = 1.0 / (rho * sqrt(c2));
   rs = rho;
-  if (drs) *drs = 1.0 / c2;
+  drs = 1.0 / c2;
   return M2C_OK;
 }
 
-__device__ inline int wave(const EosDev& q, Side& K, double p, double& f, double& df, double& rs,
-                           bool want_rho = true, double* drs = nullptr) {
-  if (q.type == M2C_EOS_SG) return wave_sg(q, K, p, f, df, rs, want_rho, drs);
-  if (q.type == M2C_EOS_MG) return wave_mg(q, K, p, f, df, rs, drs);
-  if (q.type == M2C_EOS_NASG) return wave_nasg(q, K, p, f, df, rs, drs);
-  return wave_jwl(q, K, p, f, df, rs, drs);
+// A side's wave curve at p; out of line, one copy for both sides.
+static __device__ __noinline__ int wave(const EosDev& q, Side& K, double p, Wave& w) {
+  if (q.type == M2C_EOS_SG) return wave_sg(q, K, p, w);
+  if (q.type == M2C_EOS_MG) return wave_mg(q, K, p, w);
+  if (q.type == M2C_EOS_NASG) return wave_nasg(q, K, p, w);
+  return wave_jwl(q, K, p, w);
 }
 
-// Both wave curves at p: f and f' of each side, and on request (wv) the star
-// densities behind the two waves and their slopes d rho*/dp as well.
-struct WaveVals {
-  double fL, dfL, rL, dL, fR, dfR, rR, dR;
-};
+// Density behind the wave w evaluated at p, and its slope d rho*/dp.
+__device__ inline void star_density(const EosDev& q, const Side& K, double p, const Wave& w, double& rs, double& drs) {
+  if (q.type != M2C_EOS_SG) {
+    rs = w.a;
+    drs = w.b;
+  } else if (p > K.p) {
+    const double r = (p + q.pc) * K.ipb, id = rcp_nr(fma(q.gm, r, 1.0));
+    rs = K.rho * (r + q.gm) * id;
+    drs = K.rho * fma(-q.gm, q.gm, 1.0) * (id * id) * K.ipb;
+  } else {
+    // r^(1/g) = r/(r^((g-1)/(2g)))^2
+    const double pb = p + q.pc;
+    rs = K.rho * (pb * K.ipb) * rcp_nr(w.a * w.a);
+    drs = rs * q.inv_g * rcp_nr(pb);
+  }
+}
 
-static __device__ __noinline__ int riemann_F(const EosDev& qL, Side& L, const EosDev& qR, Side& Rs, double p,
-                                double& F, double& dF, WaveVals* wv = nullptr) {
-  double fL, dfL, rL, fR, dfR, rR, dL = 0.0, dR = 0.0;
-  const bool want = wv != nullptr;
-  int st = wave(qL, L, p, fL, dfL, rL, want, want ? &dL : nullptr);
-  if (!st) st = wave(qR, Rs, p, fR, dfR, rR, want, want ? &dR : nullptr);
-  if (st) return st;
-  F = fL + fR + (Rs.u - L.u);
-  dF = dfL + dfR;
-  if (wv) *wv = WaveVals{fL, dfL, rL, dL, fR, dfR, rR, dR};
-  return M2C_OK;
+// F(p) = f_L + f_R + (u_R - u_L) of the bisection and the vacuum test.
+static __device__ __noinline__ int riemann_F(const EosDev& qL, Side& L, const EosDev& qR, Side& Rs, double p, double& F) {
+  Wave wL, wR;
+  int st = wave(qL, L, p, wL);
+  if (!st) st = wave(qR, Rs, p, wR);
+  if (!st) F = wL.f + wR.f + (Rs.u - L.u);
+  return st;
 }
 
 struct RiemannOut {
   double p, u, rhoL, rhoR;
 };
+
+// A problem whose Newton iteration ran out of steps: the vacuum test, then
+// bisection for p* (iters counts its steps too). Then, and for a converged
+// problem with a slope that is not finite, the star state from an evaluation at p.
+static __device__ __noinline__ int riemann_finish(const EosDev& qL, Side& L, const EosDev& qR, Side& Rs, double plow,
+                                                  bool vacuum_test, bool conv, double p, RiemannOut& out, int& iters) {
+  int st;
+  double F;
+  if (!conv) {
+    ++iters;
+    if (vacuum_test) {
+      st = riemann_F(qL, L, qR, Rs, plow, F);
+      if (st) return st;
+      if (F >= 0.0) return M2C_EVACUUM;
+    }
+    double a = plow, b = fmax(L.p, Rs.p);
+    if (!isfinite(a)) {
+      a = fmin(L.p, Rs.p);
+      for (int k = 0; k < kBisectCap; ++k) {
+        st = riemann_F(qL, L, qR, Rs, a, F);
+        if (st) return st;
+        if (F < 0.0) break;
+        a = a - 2.0 * fabs(a) - 1.0;
+      }
+    }
+    for (int k = 0; k < kBisectCap; ++k) {
+      st = riemann_F(qL, L, qR, Rs, b, F);
+      if (st) return st;
+      if (F > 0.0) break;
+      b = 2.0 * b + fabs(b) + 1.0;
+    }
+    bool ok = false;
+    for (int k = 0; k < kBisectCap; ++k) {
+      double m = 0.5 * (a + b);
+      st = riemann_F(qL, L, qR, Rs, m, F);
+      if (st) return st;
+      if (F < 0.0) a = m; else b = m;
+      ++iters;
+      if (b - a <= 1e-14 * fmax(fabs(a), fabs(b))) { ok = true; break; }
+    }
+    if (!ok) return M2C_ENOCONV;
+    p = 0.5 * (a + b);
+  }
+  Wave wL, wR;
+  double d;
+  st = wave(qL, L, p, wL);
+  if (!st) st = wave(qR, Rs, p, wR);
+  if (st) return st;
+  out.p = p;
+  out.u = 0.5 * (L.u + Rs.u) + 0.5 * (wR.f - wL.f);
+  star_density(qL, L, p, wL, out.rhoL, d);
+  star_density(qR, Rs, p, wR, out.rhoR, d);
+  return M2C_OK;
+}
 
 // Solves the 1D problem between (rho, u, p) states; returns a status and the
 // Newton/bisection iteration count. p_start: a start of the Newton iteration
@@ -452,8 +539,7 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
   if (!make_side(qL, rl, ul, pl, L) || !make_side(qR, rr, ur, pr, Rs)) return M2C_ENONPHYS;
   const double plow = fmax(eos_plow(qL), eos_plow(qR));
   fix_substeps(qL, L, qR, Rs, plow);
-  double F, dF;
-  int st;
+  int st = M2C_OK;
   // vacuum test (F(p_low) >= 0); both wave curves increase with p and vanish at
   // their side's pressure, so F(p_low) <= u_R - u_L and the test is only made
   // when u_R - u_L >= 0; no vacuum test with a JWL side (its rarefaction needs
@@ -470,77 +556,41 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
     if (!(gap > 0.0)) gap = fmax(L.p, Rs.p) - plow;
     p = plow + 1e-3 * gap;
   }
-  int it;
-  bool conv = false;
-  // every evaluation also returns the star densities, so that the solution
-  // follows from the last one to first order in its step (at most the
-  // tolerance: the error is of the order of its square) instead of from one
-  // more evaluation
-  WaveVals wv{};
-  double p_last = 0.0;
-  for (it = 1; it <= kNewtonCap; ++it) {
-    st = riemann_F(qL, L, qR, Rs, p, F, dF, &wv);
-    if (st) return st;
-    double pn = p - F / dF;
+  // the solution follows from the last evaluation to first order in its step (at
+  // most the tolerance: the error is of the order of its square) instead of from
+  // one more evaluation
+  Wave wL{}, wR{};
+  double p_last = p;
+  bool conv = false, more = true;
+  int it = 0;
+  while (more) {
+    ++it;
+    st = wave(qL, L, p, wL);
+    const int sr = wave(qR, Rs, p, wR);
+    if (!st) st = sr;
+    double pn = p - div_nr(wL.f + wR.f + (Rs.u - L.u), wL.df + wR.df);
     if (!(pn > plow)) pn = 0.5 * (p + plow);
-    bool small = fabs(pn - p) <= kNewtonTol * fabs(pn);
+    conv = !st && fabs(pn - p) <= kNewtonTol * fabs(pn);
     p_last = p;
     p = pn;
-    if (small) { conv = true; break; }
+    more = !st && !conv && it < kNewtonCap;
   }
-  if (!conv) {
-    if (vacuum_test) {
-      st = riemann_F(qL, L, qR, Rs, plow, F, dF);
-      if (st) return st;
-      if (F >= 0.0) return M2C_EVACUUM;
-    }
-    double a = plow, b = fmax(L.p, Rs.p);
-    if (!isfinite(a)) {
-      a = fmin(L.p, Rs.p);
-      for (int k = 0; k < kBisectCap; ++k) {
-        st = riemann_F(qL, L, qR, Rs, a, F, dF);
-        if (st) return st;
-        if (F < 0.0) break;
-        a = a - 2.0 * fabs(a) - 1.0;
-      }
-    }
-    for (int k = 0; k < kBisectCap; ++k) {
-      st = riemann_F(qL, L, qR, Rs, b, F, dF);
-      if (st) return st;
-      if (F > 0.0) break;
-      b = 2.0 * b + fabs(b) + 1.0;
-    }
-    bool ok = false;
-    for (int k = 0; k < kBisectCap; ++k) {
-      double m = 0.5 * (a + b);
-      st = riemann_F(qL, L, qR, Rs, m, F, dF);
-      if (st) return st;
-      if (F < 0.0) a = m; else b = m;
-      ++it;
-      if (b - a <= 1e-14 * fmax(fabs(a), fabs(b))) { ok = true; break; }
-    }
-    if (!ok) return M2C_ENOCONV;
-    p = 0.5 * (a + b);
-  }
-  if (conv && isfinite(wv.dfL) && isfinite(wv.dfR) && isfinite(wv.dL) && isfinite(wv.dR)) {
-    const double d = p - p_last;
-    out.p = p;
-    out.u = 0.5 * (L.u + Rs.u) + 0.5 * (wv.fR - wv.fL) + 0.5 * (wv.dfR - wv.dfL) * d;
-    out.rhoL = wv.rL + wv.dL * d;
-    out.rhoR = wv.rR + wv.dR * d;
-    iters = it;
-    return M2C_OK;
-  }
-  double fL, dfL, rL, fR, dfR, rR;
-  st = wave(qL, L, p, fL, dfL, rL);
-  if (!st) st = wave(qR, Rs, p, fR, dfR, rR);
   if (st) return st;
-  out.p = p;
-  out.u = 0.5 * (L.u + Rs.u) + 0.5 * (fR - fL);
-  out.rhoL = rL;
-  out.rhoR = rR;
-  iters = it;
-  return M2C_OK;
+  if (conv && isfinite(wL.df) && isfinite(wR.df)) {
+    double rL, dL, rR, dR;
+    star_density(qL, L, p_last, wL, rL, dL);
+    star_density(qR, Rs, p_last, wR, rR, dR);
+    if (isfinite(dL) && isfinite(dR)) {
+      const double d = p - p_last;
+      out.p = p;
+      out.u = 0.5 * (L.u + Rs.u) + 0.5 * (wR.f - wL.f) + 0.5 * (wR.df - wL.df) * d;
+      out.rhoL = rL + dL * d;
+      out.rhoR = rR + dR * d;
+      iters = it;
+      return M2C_OK;
+    }
+  }
+  return riemann_finish(qL, L, qR, Rs, plow, vacuum_test, conv, p, out, iters = it);
 }
 
 // ---------------------------------------------------------------------------
@@ -741,9 +791,12 @@ static __device__ __noinline__ int riemann_solve_mixed(const EosP<float>& qLf, c
     fix_substeps(qL, L, qR, Rs, plow);
     double p = f2d(p32);
     for (int k = 0; k < 2; ++k) {
-      double fL, dfL, rL, dL = 0.0, fR, dfR, rR, dR = 0.0;
-      if (!(p > plow) || wave(qL, L, p, fL, dfL, rL, true, &dL) || wave(qR, Rs, p, fR, dfR, rR, true, &dR)) break;
-      const double F = fL + fR + (Rs.u - L.u), dF = dfL + dfR;
+      Wave wL, wR;
+      double rL, dL, rR, dR;
+      if (!(p > plow) || wave(qL, L, p, wL) || wave(qR, Rs, p, wR)) break;
+      star_density(qL, L, p, wL, rL, dL);
+      star_density(qR, Rs, p, wR, rR, dR);
+      const double F = wL.f + wR.f + (Rs.u - L.u), dF = wL.df + wR.df;
       const double dp = -F / dF;
       // a slope that is not finite (a wave of rounding-level strength on a
       // shock curve) leaves the problem to the FP64 iteration
@@ -752,7 +805,7 @@ static __device__ __noinline__ int riemann_solve_mixed(const EosP<float>& qLf, c
         break;
       if (k == 1 || fabs(dp) <= 1e-9 * fabs(p)) {
         out.p = p + dp;
-        out.u = 0.5 * (L.u + Rs.u) + 0.5 * (fR - fL) + 0.5 * (dfR - dfL) * dp;
+        out.u = 0.5 * (L.u + Rs.u) + 0.5 * (wR.f - wL.f) + 0.5 * (wR.df - wL.df) * dp;
         out.rhoL = rL + dL * dp;
         out.rhoR = rR + dR * dp;
         iters = it32 + 1 + k;

@@ -78,17 +78,23 @@ __device__ __forceinline__ bool fiver_face_fluxes(const EosP<R>& qa, const EosP<
   return ok;
 }
 
-// One warp-sized block per 32 faces, so that the few warps of a typical
-// interface spread evenly over the SMs (each is FP64-pipe bound).
+// Warp-sized blocks, so that the warps of an interface spread evenly over the
+// SMs. A warp's FP64 instruction holds its scheduler's FP64 unit for 64 cycles
+// whatever the number of active lanes, and a warp takes every path that one of
+// its lanes takes: while there are fewer faces than schedulers x 32 lanes
+// (`units` schedulers, shared by the launch's grids), a warp takes only so many
+// faces that every scheduler gets one warp; with more faces, all 32 lanes.
 constexpr int kFiverThreads = 32;
-__global__ void __launch_bounds__(kFiverThreads, 1) k_fiver(const Grid* __restrict__ grids, int mode) {
+__global__ void __launch_bounds__(kFiverThreads, 1) k_fiver(const Grid* __restrict__ grids, int mode, int units) {
   const Grid& G = grids[blockIdx.y];
   Ctrl* ctrl = G.ctrl;
   const int slot = list_slot(mode);
   const int n = min(ctrl->nface[slot], G.face_cap);
   const double* __restrict__ Ws = stage_W(G, mode);
   const long long N = G.N;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  const int per = min(kFiverThreads, max(1, (int)(((long long)n * gridDim.y + units - 1) / units)));
+  if ((int)threadIdx.x >= per) return;
+  for (int i = blockIdx.x * per + threadIdx.x; i < n; i += gridDim.x * per) {
     const IfFace f = G.faces[i];
     const long long ca = f.cell;
     const int ix = (int)(ca % G.nx), iy = (int)((ca / G.nx) % G.ny), iz = (int)(ca / ((long long)G.nx * G.ny));
@@ -533,12 +539,14 @@ __global__ void k_shock_state(EosDev q, double rho, double u, double p, double p
     *status = M2C_EINVAL;
     return;
   }
-  double f, df, rs;
-  const int st = wave(q, K, p1, f, df, rs);
+  Wave w;
+  double rs, drs;
+  const int st = wave(q, K, p1, w);
   *status = st;
   if (st) return;
+  star_density(q, K, p1, w, rs, drs);
   out[0] = rs;
-  out[1] = K.u + f;
+  out[1] = K.u + w.f;
   out[2] = (rs * out[1] - K.rho * K.u) / (rs - K.rho);
 }
 
@@ -884,6 +892,16 @@ cudaError_t record_pair(StageEvents* pe, bool start, cudaStream_t s, int kind = 
   return e;
 }
 
+// Launch of k_fiver: blocks for twice the faces of a surface across the largest
+// grid (N^(2/3); a shock-bubble of radius 0.15 to 0.25 has about as many), at
+// least one per scheduler; more faces go round the block loop again.
+void launch_fiver(const Grid* grids, int ngrid, long long nmax, int mode, cudaStream_t s) {
+  const long long units = 4ll * sm_count();
+  const double surface = std::cbrt((double)nmax) * std::cbrt((double)nmax);
+  const long long nb = std::max(units, std::min(16 * units, (long long)(2.0 * surface / kFiverThreads) + 1));
+  k_fiver<<<dim3((unsigned)nb, (unsigned)ngrid), kFiverThreads, 0, s>>>(grids, mode, (int)units);
+}
+
 // reinit: enqueue the reinitialisation kernels (each grid decides on the device
 // whether its own step is due); reinit_iters: the largest iteration count.
 // rk: the Runge-Kutta scheme of all grids (Sec. 4.3); gen: launch the general
@@ -893,7 +911,6 @@ cudaError_t enqueue_step(const Grid* dev_grids, const long long* dev_tiles, int 
                          StageEvents* pe = nullptr, int rk = 2, bool gen = false, bool band = false) {
   cudaError_t e;
   const dim3 lg((unsigned)(2 * sm_count()), (unsigned)ngrid);
-  const dim3 fg((unsigned)(8 * sm_count()), (unsigned)ngrid);
 #define M2C_TIMED(kind, launch)                                     \
   do {                                                              \
     if ((e = record_pair(pe, true, s, kind)) != cudaSuccess) return e; \
@@ -909,7 +926,7 @@ cudaError_t enqueue_step(const Grid* dev_grids, const long long* dev_tiles, int 
   for (int stage = 0; stage < nstage; ++stage) {
     const int mode = modes[stage];
     M2C_TIMED(kKStage, e = launch_stage(prec, dev_grids, dev_tiles, ngrid, ntiles, mode, lp, s, gen); if (e) return e);
-    M2C_TIMED(kKFiver, (k_fiver<<<fg, kFiverThreads, 0, s>>>(dev_grids, mode)));
+    M2C_TIMED(kKFiver, launch_fiver(dev_grids, ngrid, nmax, mode, s));
     M2C_TIMED(kKFinish, (k_finish<<<lg, 128, 0, s>>>(dev_grids, mode)));
   }
   if (rk == 1) {
@@ -1486,7 +1503,7 @@ m2c_status m2c_residual(m2c_ctx* c, double* R, double* L) {
                                c->stream, c->host.general != 0);
   if (e == cudaSuccess) {
     const dim3 lg((unsigned)(2 * sm_count()), 1);
-    k_fiver<<<dim3((unsigned)(8 * sm_count()), 1), kFiverThreads, 0, c->stream>>>(c->dev_grid, kResidual);
+    launch_fiver(c->dev_grid, 1, c->host.N, kResidual, c->stream);
     k_finish<<<lg, 128, 0, c->stream>>>(c->dev_grid, kResidual);
     e = cudaGetLastError();
   }
@@ -1770,7 +1787,7 @@ m2c_status m2c_residual_noalloc(int nx, int ny, int nz, double h, const int bc[6
   if (e == cudaSuccess) e = launch_stage(precision, dg, dt, 1, tiles[1], kResidual, lp, s);
   if (e == cudaSuccess) {
     const dim3 lg((unsigned)(2 * sm_count()), 1);
-    k_fiver<<<dim3((unsigned)(8 * sm_count()), 1), kFiverThreads, 0, s>>>(dg, kResidual);
+    launch_fiver(dg, 1, N, kResidual, s);
     k_finish<<<lg, 128, 0, s>>>(dg, kResidual);
     e = cudaGetLastError();
   }
