@@ -33,10 +33,11 @@ struct Side {
   double iv, ic2, hp, hr, hd;
   int nrk;  // RK4 substeps of this side's MG rarefaction curve in one problem; 0: per evaluation
   // MG: spacing of the problem's fixed RK4 nodes p_K - i dnode (0: none), and the
-  // isentrope state (rho, f) after the first mbase full substeps, kept between the
-  // evaluations of one problem (nearby pressures share their nodes)
+  // isentrope states (rho, f) after the first mbase and mbase - 1 full substeps, kept
+  // between the evaluations of one problem (nearby pressures share their nodes; the
+  // iteration may step back over one)
   int mbase;
-  double dnode, idnode, dspan, rbase, fbase;  // dspan = nrk dnode, the span bound the nodes cover
+  double dnode, idnode, dspan, rbase, fbase, rprev, fprev;  // dspan = nrk dnode, the span bound the nodes cover
 };
 
 __device__ inline bool make_side(const EosDev& q, double rho, double u, double p, Side& K) {
@@ -63,8 +64,8 @@ __device__ inline bool make_side(const EosDev& q, double rho, double u, double p
     K.mbase = 0;
     K.dnode = 0.0;
     K.dspan = 0.0;
-    K.rbase = rho;
-    K.fbase = 0.0;
+    K.rbase = K.rprev = rho;
+    K.fbase = K.fprev = 0.0;
   }
   return true;
 }
@@ -102,7 +103,8 @@ __device__ inline int jwl_substeps(double pK, double p_lo) {
 // (a shock on the other side J keeps p* above p_J; a rarefaction there too
 // keeps p* above p_ac, since each rarefaction curve lies below its acoustic
 // tangent). Written without contracted multiply-adds.
-__device__ inline void fix_substeps(const EosDev& qL, Side& L, const EosDev& qR, Side& Rs, double plow) {
+// Returns p_ac.
+__device__ inline double fix_substeps(const EosDev& qL, Side& L, const EosDev& qR, Side& Rs, double plow) {
   const double ZL = __dmul_rn(L.rho, L.c), ZR = __dmul_rn(Rs.rho, Rs.c);
   const double num = __dsub_rn(__dadd_rn(__dmul_rn(ZR, L.p), __dmul_rn(ZL, Rs.p)),
                                __dmul_rn(__dmul_rn(ZL, ZR), __dsub_rn(Rs.u, L.u)));
@@ -120,6 +122,7 @@ __device__ inline void fix_substeps(const EosDev& qL, Side& L, const EosDev& qR,
   if (qR.type == M2C_EOS_MG) mg_nodes(qR, Rs, loR);
   if (qL.type == M2C_EOS_JWL) L.nrk = jwl_substeps(L.p, loL);
   if (qR.type == M2C_EOS_JWL) Rs.nrk = jwl_substeps(Rs.p, loR);
+  return pac;
 }
 
 // One side's wave curve at a pressure: f and f', and what the star density
@@ -191,26 +194,26 @@ __device__ inline int mg_hugoniot(const EosDev& q, Side& K, double p, double& rh
 }
 
 // Right-hand side of the MG isentrope. With d = rho - rho0 and q = rho - s d
-// (1 - s eta = q/rho), the sound speed of the compression branch is
-//   rho^2 c^2 = K0 rho0 A,  A = (rho + (s - G0) d) rho^2/q^3 + (G0/K0) p,
-// and that of the tension branch A = (rho - G0 d)/rho + (G0/K0) p (s = 0, the
-// factor 1/rho instead of rho^2/q^3). So d rho/dp = 1/c^2 = (rho y)^2/(K0 rho0)
-// and df/dp = 1/(rho c) = y/(K0 rho0)^(1/2) with y = A^(-1/2): 17 FP64
-// instructions with one reciprocal and one root (35 through the general e and
-// c^2); the constant factors sit in the substep lengths. gp = (G0/K0) p. ok is
-// cleared outside the EOS domain (rho <= 0, eta >= 1/s, c^2 <= 0). A finite
-// tension cutoff takes the general sound speed.
-__device__ inline void mg_rhs(const EosDev& q, double gp, double rho, double& kr, double& y, bool& ok) {
+// (1 - s eta = q/rho) the sound speed of the compression branch is
+//   rho^2 c^2 = K0 rho0 A,  A = n rho^2/q^3 + g,  n = rho + (s - G0) d,  g = (G0/K0) p,
+// and the tension branch has the same form with q = rho (s = 0). d rho/dp = 1/c^2 =
+// (rho y)^2/(K0 rho0) and df/dp = 1/(rho c) = y/(K0 rho0)^(1/2) with y = A^(-1/2) =
+// q^2 (q (n rho^2 + g q^3))^(-1/2): 16 FP64 instructions with one root and no
+// division (35 through the general e and c^2); the constant factors sit in the
+// substep lengths. ok is cleared outside the EOS domain (rho <= 0, eta >= 1/s,
+// c^2 <= 0). Below a finite tension cutoff A = g - (G0/K0) p_min.
+__device__ inline void mg_rhs(const EosDev& q, double g, double rho, double& kr, double& y, bool& ok) {
   const double d = rho - q.rho0;
   const bool comp = gt0(d);
-  const double qq = fma(comp ? -q.s : 0.0, d, rho), n = fma(comp ? q.sG : -q.G0, d, rho);
-  ok = ok && gt0(rho) && nr_range_pos(qq);
-  const double iq = rcp_nr_in_range(qq);
-  const double t = comp ? rho * iq : 1.0;
-  double A = fma(n, t * t * iq, gp);
-  if (q.eta_min > -INFINITY && q.rho0 * rcp_nr(rho) > 1.0 - q.eta_min) A = gp - q.gk * q.pmin;
-  ok = ok && nr_range_pos(A);
-  y = rsqrt_nr_in_range(A);
+  double qq = fma(comp ? -q.s : 0.0, d, rho);
+  const double n = fma(comp ? q.sG : -q.G0, d, rho);
+  double C = qq * fma(n, rho * rho, g * (qq * qq * qq)), q2 = qq * qq;
+  if (q.eta_min > -INFINITY && q.rho0 * rcp_nr(rho) > 1.0 - q.eta_min) {
+    C = g - q.gk * q.pmin;
+    q2 = 1.0;
+  }
+  ok = ok && gt0(rho) && gt0(qq) && nr_range_pos(C);
+  y = q2 * rsqrt_nr_in_range(C);
   const double ry = rho * y;
   kr = ry * ry;
 }
@@ -230,13 +233,14 @@ __device__ inline void mg_rk4_substep(const EosDev& q, double pi, double hs, dou
 
 // MG wave curve. Rarefaction: the isentrope integrated by classical RK4 in p;
 // inside a problem's span bound on the fixed nodes p_K - i dnode (full substeps
-// down to the last node above p, resumed from the node reached by an earlier
-// evaluation of the problem when it lies at or below, then one partial substep
-// to p): the curve is continuous and smooth in p; beyond the bound, and for a
-// wave evaluated alone, equal substeps over p_K - p. Both are one loop, so that
-// the lanes of a warp take their substeps together. The node arithmetic is
-// written without contracted multiply-adds, so that it takes the same nodes as
-// the oracle.
+// down to the last node above p, resumed from a node reached by an earlier
+// evaluation of the problem, then one partial substep to p): the curve is
+// continuous and smooth in p. An iterate less than a node spacing beyond the bound
+// takes all nodes and the partial substep too (the root lies inside the bound, and
+// the nodes serve the next iterate); further beyond, and for a wave evaluated
+// alone, equal substeps over p_K - p. All are one loop, so that the lanes of a
+// warp take their substeps together. The node arithmetic is written without
+// contracted multiply-adds, so that it takes the same nodes as the oracle.
 __device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
   int st = M2C_OK;
   if (p == K.p) {
@@ -255,17 +259,21 @@ __device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
     w.b = drdp;
   } else {
     const double dp = __dsub_rn(K.p, p);
-    const bool within = K.nrk > 1 && K.dnode > 0.0 && dp < K.dspan;
+    const bool within = K.nrk > 1 && K.dnode > 0.0 && dp < K.dspan + K.dnode;
     double rho = K.rho, fv = 0.0, gap = 0.0, last = dp;
     int i = 0, m = 0;
     if (within) {
       const double m0 = dp * K.idnode;
       m = (int)floor(fma(fma(-K.dnode, m0, dp), K.idnode, m0));  // the IEEE quotient dp/dnode
-      if (m > K.nrk - 1) m = K.nrk - 1;
-      if (K.mbase <= m) {  // resume from the deepest node, unless an earlier evaluation went past m
+      m = min(m, dp < K.dspan ? K.nrk - 1 : K.nrk);
+      if (K.mbase <= m) {
         i = K.mbase;
         rho = K.rbase;
         fv = K.fbase;
+      } else if (K.mbase == m + 1) {
+        i = m;
+        rho = K.rprev;
+        fv = K.fprev;
       }
       gap = K.dnode;
     } else {
@@ -279,14 +287,23 @@ __device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
       }
     }
     bool ok = true;
-    for (; i < m; ++i) mg_rk4_substep(q, __dsub_rn(K.p, __dmul_rn((double)i, gap)), -gap, rho, fv, ok);
-    const double pm = __dmul_rn((double)m, gap);
-    if (within) {
-      K.mbase = m;
-      K.rbase = rho;
-      K.fbase = fv;
-      last = __dsub_rn(dp, pm);
+    if (i < m) {
+      double rp = rho, fp = fv;
+      for (; i < m; ++i) {
+        rp = rho;
+        fp = fv;
+        mg_rk4_substep(q, __dsub_rn(K.p, __dmul_rn((double)i, gap)), -gap, rho, fv, ok);
+      }
+      if (within) {
+        K.mbase = m;
+        K.rbase = rho;
+        K.fbase = fv;
+        K.rprev = rp;
+        K.fprev = fp;
+      }
     }
+    const double pm = __dmul_rn((double)m, gap);
+    if (within) last = __dsub_rn(dp, pm);
     if (last > 0.0) mg_rk4_substep(q, __dsub_rn(K.p, pm), -last, rho, fv, ok);
     double k, y;
     mg_rhs(q, q.gk * p, rho, k, y, ok);
@@ -526,19 +543,69 @@ static __device__ __noinline__ int riemann_finish(const EosDev& qL, Side& L, con
   return M2C_OK;
 }
 
+// One side in the FP32 start below: a stiffened gas, or an MG material taken as one
+// with the exponent n = 4 s - 1 of its isentrope near the reference state and the
+// side's sound speed.
+struct GuessSide {
+  float rho, p, c, n, pb;
+};
+__device__ inline GuessSide guess_side(const EosDev& q, const Side& K) {
+  const float rho = d2f(K.rho), c = d2f(K.c);
+  const bool sg = q.type == M2C_EOS_SG;
+  const float n = sg ? d2f(q.g) : fmaf(4.0f, d2f(q.s), -1.0f);
+  return {rho, d2f(K.p), c, n, sg ? d2f(K.pb) : __fdividef(rho * c * c, n)};
+}
+__device__ inline void guess_wave(const GuessSide& K, float p, float& f, float& df) {
+  const float dp = p - K.p, m = __fdividef(K.n - 1.0f, K.n + 1.0f);
+  if (dp > 0.0f) {
+    const float id = __fdividef(1.0f, fmaf(1.0f + m, K.pb, dp)), sq = sqrtf((1.0f - m) * __fdividef(id, K.rho));
+    f = dp * sq;
+    df = sq * fmaf(-0.5f * dp, id, 1.0f);
+  } else {
+    const float r = fmaxf(1.0f + __fdividef(dp, K.pb), 1e-6f);
+    const float w = __powf(r, __fdividef(0.5f * (K.n - 1.0f), K.n));
+    f = __fdividef(2.0f * K.c, K.n - 1.0f) * (w - 1.0f);
+    df = __fdividef(w, r * K.rho * K.c);
+  }
+}
+
+// Start of the Newton iteration of a face without a previous star pressure: p* to
+// a few per cent from eight FP32 Newton steps on closed-form curves, from the
+// acoustic pressure p_ac. NaN where that fails. The PVRS estimate is far off p*
+// when the sides' impedances differ (water against air) and takes 13
+// iterations, three of them over the whole isentrope; one such face held up its
+// launch (1.51 against 0.59 ms in the late shock-bubble, 131x67x45).
+static __device__ __noinline__ double start_guess(const EosDev& qL, const Side& L, const EosDev& qR, const Side& Rs,
+                                                  double plow, double pac) {
+  if ((qL.type != M2C_EOS_SG && qL.type != M2C_EOS_MG) || (qR.type != M2C_EOS_SG && qR.type != M2C_EOS_MG)) return NAN;
+  const GuessSide gl = guess_side(qL, L), gr = guess_side(qR, Rs);
+  const float du = d2f(Rs.u - L.u), low = d2f(fmax(plow, -1e30));
+  float p = fmaxf(d2f(pac), fmaf(1e-3f, fminf(gl.p, gr.p) - low, low));
+  for (int k = 0; k < 8; ++k) {
+    float fl, dl, fr, dr;
+    guess_wave(gl, p, fl, dl);
+    guess_wave(gr, p, fr, dr);
+    const float pn = p - __fdividef(fl + fr + du, dl + dr);
+    p = pn > low ? pn : fmaf(0.5f, p - low, low);
+  }
+  return p > low && p < INFINITY ? f2d(p) : (double)NAN;
+}
+
 // Solves the 1D problem between (rho, u, p) states; returns a status and the
 // Newton/bisection iteration count. p_start: a start of the Newton iteration
 // (the FIVER kernel passes the same face's star pressure of its previous
 // solve); NaN, or a value not above the lowest admissible pressure, takes the
-// PVRS estimate. The root and the stopping rule do not depend on the start.
+// PVRS estimate, or, with `guess`, start_guess() where the PVRS estimate and the
+// acoustic pressure differ by more than 5 %. The root and the stopping rule do
+// not depend on the start.
 static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, double ul, double pl, const EosDev& qR, double rr,
                                     double ur, double pr, RiemannOut& out, int& iters,
-                                    double p_start = NAN) {
+                                    double p_start = NAN, bool guess = false) {
   Side L, Rs;
   iters = 0;
   if (!make_side(qL, rl, ul, pl, L) || !make_side(qR, rr, ur, pr, Rs)) return M2C_ENONPHYS;
   const double plow = fmax(eos_plow(qL), eos_plow(qR));
-  fix_substeps(qL, L, qR, Rs, plow);
+  const double pac = fix_substeps(qL, L, qR, Rs, plow);
   int st = M2C_OK;
   // vacuum test (F(p_low) >= 0); both wave curves increase with p and vanish at
   // their side's pressure, so F(p_low) <= u_R - u_L and the test is only made
@@ -550,7 +617,12 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
   const bool vacuum_test = isfinite(plow) && Rs.u - L.u >= 0.0 && qL.type != M2C_EOS_JWL && qR.type != M2C_EOS_JWL;
   double p = 0.5 * (L.p + Rs.p) - 0.125 * (Rs.u - L.u) * (L.rho + Rs.rho) * (L.c + Rs.c);
   const bool warm = p_start > plow && p_start < INFINITY;
-  if (warm) p = p_start;
+  if (warm) {
+    p = p_start;
+  } else if (guess && !(fabs(p - pac) <= 0.05 * fabs(pac))) {
+    const double pg = start_guess(qL, L, qR, Rs, plow, pac);
+    if (pg > plow) p = pg;
+  }
   if (!(p > plow)) {
     double gap = fmin(L.p, Rs.p) - plow;
     if (!(gap > 0.0)) gap = fmax(L.p, Rs.p) - plow;

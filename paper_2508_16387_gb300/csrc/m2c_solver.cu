@@ -111,8 +111,8 @@ __global__ void __launch_bounds__(kFiverThreads, 1) k_fiver(const Grid* __restri
     int its = 0;
     int st = M2C_ENONPHYS;
     // Newton starts from this face's star pressure of its last solve (the previous
-    // stage), else from the PVRS estimate; the residual alone (kResidual) always
-    // starts from PVRS
+    // stage), else from an estimate; the residual alone (kResidual) always starts
+    // from the estimate
     double* pst = (mode != kResidual && G.pstar) ? G.pstar + 3 * ca + d : nullptr;
     const double p_start = pst ? *pst : (double)NAN;
     if (ok) {
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kFiverThreads, 1) k_fiver(const Grid* __restri
         st = riemann_solve_mixed(G.eosf[mirror ? ib : ia], q0, P0[0], sgn * P0[1 + d], P0[4], G.eosf[mirror ? ia : ib], q1,
                                  P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start);
       else
-        st = riemann_solve(q0, P0[0], sgn * P0[1 + d], P0[4], q1, P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start);
+        st = riemann_solve(q0, P0[0], sgn * P0[1 + d], P0[4], q1, P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start, true);
       if (pst && st == M2C_OK) *pst = rs.p;
       if (mirror) {
         const double r = rs.rhoL;
