@@ -57,11 +57,12 @@ __device__ __forceinline__ bool cons_to_prim_v(const EosP<R>& q, const EosDev& q
     const double inv = rrcp<double>(rho);
     const double u = m1 * inv, v = m2 * inv, w = m3 * inv;
     const double ke = 0.5 * ((m1 * u + m2 * v) + m3 * w);
-    const double e = (E - ke) * inv;
     double p = 0.0;
-    const bool ok = eos_p<double, EXT, T>(q, rho, inv, e, p);
+    bool ok = true;
+    if (eos_is<T>(q, M2C_EOS_SG)) p = fma(q.gm1, E - ke, -q.gpc);
+    else ok = eos_p<double, EXT, T>(q, rho, inv, (E - ke) * inv, p);
     P[0] = rho; P[1] = u; P[2] = v; P[3] = w; P[4] = p;
-    return ok && rho > 0.0;
+    return ok && gt0(rho);
   } else {
     const double x[4] = {rho, m1, m2, m3};
     float y[4];
