@@ -204,9 +204,9 @@ m2c_status m2c_set_riemann_start(m2c_ctx* ctx, int fp32_start);
  * not depend on the tiling (bitwise); M2C_MIXED results agree to FP32 rounding
  * (FP32 multiply-adds may be contracted differently in the code that opens a
  * z-chunk and in the kernels of other tile heights). Default: the
- * rows (8, or 16 for M2C_MIXED and 4 for M2C_FP64) and tile_z with the smaller
- * estimated time for the grid's size: short tiles that give every SM work on a
- * small grid, longer ones on a large grid. */
+ * rows (8, or 4 for M2C_FP64 where 8 give too few tiles) and tile_z with the
+ * smaller estimated time for the grid's size: short tiles that give every SM work
+ * on a small grid, longer ones on a large grid. */
 m2c_status m2c_set_tiling(m2c_ctx* ctx, int tile_rows, int tile_z);
 
 /* Borrows the device arrays W (5N doubles, the conserved state of Sec. 3.2,

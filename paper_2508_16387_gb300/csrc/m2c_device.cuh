@@ -16,6 +16,19 @@ namespace m2c {
 __device__ __forceinline__ double gld(const double* p) { return __ldg(p); }
 __device__ __forceinline__ void gst(double* p, double v) { __stwb(p, v); }
 
+// Starts bringing the 32 values from a[i] (fewer at the array's end, n values) into
+// L2: a bulk prefetch of whole 16-byte units inside the array. The plane loads of
+// the bulk kernel wait for DRAM otherwise (their loads, conversions and staging
+// alone took 0.59 ms at 256^3, five times what HBM needs).
+__device__ __forceinline__ void prefetch_row(const double* a, long long n, int i) {
+  const unsigned long long p = (reinterpret_cast<unsigned long long>(a + i) + 15ull) & ~15ull;
+  const unsigned long long e = reinterpret_cast<unsigned long long>(a + n) & ~15ull;
+  if (p < e) {
+    const unsigned bytes = (unsigned)(e - p < 256ull ? e - p : 256ull);
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Conservative -> primitive
 // ---------------------------------------------------------------------------
@@ -28,26 +41,38 @@ __device__ __forceinline__ void gst(double* p, double v) { __stwb(p, v); }
 //
 // cons_to_prim_f is the mixed path after the loads: rho, rho u, rho v, rho w
 // already rounded to binary32 (rf, f1, f2, f3), rho and rho E in binary64.
+//
+// In two parts, so that only the pressure depends on the material: the velocities
+// (into P[1..3]; returns rho e) and the pressure.
+__device__ __forceinline__ double prim_velocities_f(float inv, float f1, float f2, float f3, double E, float P[5]) {
+  P[1] = __fmul_rn(f1, inv);
+  P[2] = __fmul_rn(f2, inv);
+  P[3] = __fmul_rn(f3, inv);
+  const float ke = 0.5f * __fmaf_rn(f3, P[3], __fmaf_rn(f1, P[1], __fmul_rn(f2, P[2])));
+  return E - f2d(ke);
+}
+template <bool EXT = false, int T = -1>
+__device__ __forceinline__ bool prim_pressure_f(const EosP<float>& q, const EosDev& qd, double rho, float rf, float inv,
+                                                double rhoe, float& p) {
+  if (eos_is<T>(q, M2C_EOS_SG)) {
+    p = d2f(fma(qd.gm1, rhoe, -qd.gpc));
+    return true;
+  }
+  if (EXT && eos_is<T>(q, M2C_EOS_NASG)) {
+    const double d = 1.0 - rho * qd.b;
+    p = d2f(div_nr(qd.gm1 * (rhoe - rho * qd.ec), d) - qd.gpc);
+    return d > 0.0;
+  }
+  p = 0.0f;
+  return eos_p<float, EXT, T>(q, rf, inv, __fmul_rn(d2f(rhoe), inv), p);
+}
 template <bool EXT = false, int T = -1>
 __device__ __forceinline__ bool cons_to_prim_f(const EosP<float>& q, const EosDev& qd, double rho, float rf, float f1,
                                                float f2, float f3, double E, float P[5]) {
   const float inv = rrcp<float>(rf);
-  const float u = f1 * inv, v = f2 * inv, w = f3 * inv;
-  const float ke = 0.5f * ((f1 * u + f2 * v) + f3 * w);
-  const double rhoe = E - f2d(ke);
-  float p = 0.0f;
-  bool ok = true;
-  if (eos_is<T>(q, M2C_EOS_SG)) {
-    p = d2f(qd.gm1 * rhoe - qd.gpc);
-  } else if (EXT && eos_is<T>(q, M2C_EOS_NASG)) {
-    const double d = 1.0 - rho * qd.b;
-    ok = d > 0.0;
-    p = d2f(div_nr(qd.gm1 * (rhoe - rho * qd.ec), d) - qd.gpc);
-  } else {
-    ok = eos_p<float, EXT, T>(q, rf, inv, d2f(rhoe) * inv, p);
-  }
-  P[0] = rf; P[1] = u; P[2] = v; P[3] = w; P[4] = p;
-  return ok && gt0(rho);
+  P[0] = rf;
+  const double rhoe = prim_velocities_f(inv, f1, f2, f3, E, P);
+  return prim_pressure_f<EXT, T>(q, qd, rho, rf, inv, rhoe, P[4]) && gt0(rho, rf);
 }
 
 template <typename R, bool EXT = false, int T = -1>
@@ -55,12 +80,12 @@ __device__ __forceinline__ bool cons_to_prim_v(const EosP<R>& q, const EosDev& q
                                                double m3, double E, R P[5]) {
   if constexpr (sizeof(R) == 8) {
     const double inv = rrcp<double>(rho);
-    const double u = m1 * inv, v = m2 * inv, w = m3 * inv;
-    const double ke = 0.5 * ((m1 * u + m2 * v) + m3 * w);
+    // fused operations written out: the same bits in every kernel (a time step taken from a
+    // restored state repeats the one taken in the step before)
+    const double u = __dmul_rn(m1, inv), v = __dmul_rn(m2, inv), w = __dmul_rn(m3, inv);
+    const double ke = 0.5 * fma(m3, w, fma(m1, u, __dmul_rn(m2, v)));
     double p = 0.0;
-    bool ok = true;
-    if (eos_is<T>(q, M2C_EOS_SG)) p = fma(q.gm1, E - ke, -q.gpc);
-    else ok = eos_p<double, EXT, T>(q, rho, inv, (E - ke) * inv, p);
+    const bool ok = eos_p<double, EXT, T>(q, rho, inv, __dmul_rn(E - ke, inv), p);
     P[0] = rho; P[1] = u; P[2] = v; P[3] = w; P[4] = p;
     return ok && gt0(rho);
   } else {
@@ -77,13 +102,41 @@ __device__ __forceinline__ bool cons_to_prim(const EosP<R>& q, const EosDev& qd,
   return cons_to_prim_v<R, EXT>(q, qd, W[c], W[N + c], W[2 * N + c], W[3 * N + c], W[4 * N + c], P);
 }
 
+// e and c^2 of an FP32 face state (mixed path) for a material type fixed at compile
+// time: no branches, every rounding written out, so that the face states do not
+// depend on how the compiler contracts them in each kernel. False if not admissible.
+template <int T>
+__device__ __forceinline__ bool face_eos_f(const EosP<float>& q, float rho, float inv, float p, float& e, float& c2) {
+  bool ok = rho > 0.0f;
+  if constexpr (T == M2C_EOS_SG) {
+    e = __fmul_rn(__fmul_rn(p + q.gpc, q.inv_gm1), inv);
+    c2 = __fmul_rn(__fmul_rn(q.g, p + q.pc), inv);
+  } else {
+    ok = mg_e_c2_f(q, inv, p, e, c2) && ok;
+  }
+  return ok && c2 > 0.0f && c2 < INFINITY;
+}
+
+// A face state from its primitive fields and (e, c^2); the energy's kinetic part in FP32
+// with its roundings written out.
+__device__ __forceinline__ void finish_face_f(const float P[5], float e, float c2, bool ok, FaceState<float>& F) {
+  F.rho = P[0]; F.u = P[1]; F.v = P[2]; F.w = P[3]; F.p = P[4];
+  F.c = ok ? rsqrt_pos<float>(c2) : 0.0f;
+  F.E = __fmaf_rn(0.5f, __fmaf_rn(F.w, F.w, __fmaf_rn(F.u, F.u, __fmul_rn(F.v, F.v))), e);
+}
+
 template <typename R, bool EXT = false, int T = -1>
 __device__ __forceinline__ bool make_face(const EosP<R>& q, R rho, R u, R v, R w, R p, FaceState<R>& F) {
   R e = (R)0, c2 = (R)0;
   const bool ok = eos_e_c2<R, EXT, T>(q, rho, rrcp<R>(rho), p, e, c2);
-  F.rho = rho; F.u = u; F.v = v; F.w = w; F.p = p;
-  F.c = ok ? rsqrt_pos<R>(c2) : (R)0;
-  F.E = e + (R)0.5 * ((u * u + v * v) + w * w);
+  if constexpr (sizeof(R) == 4) {
+    const float P[5] = {rho, u, v, w, p};
+    finish_face_f(P, e, c2, ok, F);
+  } else {
+    F.rho = rho; F.u = u; F.v = v; F.w = w; F.p = p;
+    F.c = ok ? rsqrt_pos<R>(c2) : (R)0;
+    F.E = e + (R)0.5 * ((u * u + v * v) + w * w);
+  }
   return ok;
 }
 
@@ -129,20 +182,33 @@ __device__ __forceinline__ void cell_faces(const EosP<R>& q, const R Pm[5], cons
   Qp = Qm;
 }
 
+// The same bits.
+__device__ __forceinline__ bool same_bits(double a, double b) { return ((hi_of(a) ^ hi_of(b)) | (lo_of(a) ^ lo_of(b))) == 0u; }
+__device__ __forceinline__ bool same_bits(float a, float b) { return bits_of(a) == bits_of(b); }
+// Neither an infinity nor a NaN.
+__device__ __forceinline__ bool is_finite(double x) { return (hi_of(x) & 0x7ff00000u) != 0x7ff00000u; }
+__device__ __forceinline__ bool is_finite(float x) { return (bits_of(x) & 0x7f800000u) != 0x7f800000u; }
+
 // Wave-speed sum of a state, sum over the axes with more than one cell of
 // |V_d| + c (the CFL reading of the design notes), in precision R (the mixed
 // path takes the time step from FP32 wave speeds of the FP64 state).
 template <typename R, bool EXT = false, int T = -1>
-__device__ __forceinline__ R wave_sum_v(const Grid& g, const EosP<R>& q, const EosDev& qd, const double w[5], bool& ok) {
-  R P[5];
-  ok = cons_to_prim_v<R, EXT, T>(q, qd, w[0], w[1], w[2], w[3], w[4], P);
+__device__ __forceinline__ R wave_sum_p(const Grid& g, const EosP<R>& q, const R P[5], bool& ok) {
   R e, c2;
-  ok = ok && eos_e_c2<R, EXT, T>(q, P[0], rrcp<R>(P[0]), P[4], e, c2);
+  ok = eos_e_c2<R, EXT, T>(q, P[0], rrcp<R>(P[0]), P[4], e, c2);
   const R cs = ok ? rsqrt_pos<R>(c2) : (R)0;
   R lam = (R)0;
   if (g.active[0]) lam = lam + (fabs(P[1]) + cs);
   if (g.active[1]) lam = lam + (fabs(P[2]) + cs);
   if (g.active[2]) lam = lam + (fabs(P[3]) + cs);
+  return lam;
+}
+template <typename R, bool EXT = false, int T = -1>
+__device__ __forceinline__ R wave_sum_v(const Grid& g, const EosP<R>& q, const EosDev& qd, const double w[5], bool& ok) {
+  R P[5];
+  const bool okp = cons_to_prim_v<R, EXT, T>(q, qd, w[0], w[1], w[2], w[3], w[4], P);
+  const R lam = wave_sum_p<R, EXT, T>(g, q, P, ok);
+  ok = ok && okp;
   return lam;
 }
 

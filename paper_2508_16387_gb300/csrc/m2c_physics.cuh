@@ -120,7 +120,7 @@ __device__ __forceinline__ R rrcp(R x) {
 template <typename R>
 __device__ __forceinline__ R rsqrt_pos(R x) {  // sqrt of x > 0
   if constexpr (sizeof(R) == 8) return sqrt_nr(x);
-  else return x * rsqrtf(x);
+  else return __fmul_rn(x, rsqrtf(x));  // rounded: not contracted into the sums it enters
 }
 
 // Exact IEEE-754 binary64 <-> binary32 conversions written with 32-bit
@@ -204,6 +204,9 @@ __host__ __device__ __forceinline__ bool gt0(double x) {
   const unsigned hi = hi_of(x), lo = lo_of(x);
   return (hi - 1u < 0x7fefffffu) || (hi == 0u && lo != 0u) || (hi == 0x7ff00000u && lo == 0u);
 }
+// The same given y, x rounded to binary32: y decides unless x rounded to zero.
+__device__ __forceinline__ bool lt0(double x, float y) { return y < 0.0f || (y == 0.0f && lt0(x)); }
+__device__ __forceinline__ bool gt0(double x, float y) { return y > 0.0f || (y == 0.0f && gt0(x)); }
 
 // The cases outside the normal binary32 range (subnormal results, overflow,
 // zeros, infinities, NaNs), out of line so that the common path stays short.
@@ -272,10 +275,9 @@ inline __host__ __device__ __noinline__ double f2d_rare(float x) {
 
 __host__ __device__ __forceinline__ double f2d(float x) {
   const unsigned f = bits_of(x), a = f & 0x7fffffffu;
-  if (a - 0x00800000u < 0x7f800000u - 0x00800000u)  // normal: rebias 127 -> 1023
-    return double_of_words(((a >> 3) + (896u << 20)) | (f & 0x80000000u), a << 29);
-  if (a == 0u) return double_of_words(f, 0u);  // signed zero, inline
-  return f2d_rare(x);
+  // normal: rebias 127 -> 1023; a signed zero keeps its word; one branch for the rest
+  if (a - 0x00800000u >= 0x7f800000u - 0x00800000u && a != 0u) return f2d_rare(x);
+  return double_of_words(a == 0u ? f : ((a >> 3) + (896u << 20)) | (f & 0x80000000u), a << 29);
 }
 
 // A group of binary64 -> binary32 conversions (the plane loads of the mixed
@@ -459,11 +461,39 @@ __device__ __forceinline__ bool eos_is(const EosP<R>& q, int type) {
   else return q.type == type;
 }
 
+// MG p(rho, e) in FP32 (mixed path), without a branch between compression and tension,
+// every rounding written out (those of mg_ref and the general form below).
+__device__ __forceinline__ bool mg_p_f(const EosP<float>& q, float inv_rho, float e, float& p) {
+  const float eta = __fmaf_rn(-q.rho0, inv_rho, 1.0f);
+  const bool comp = eta > 0.0f;
+  const float id = comp ? __fdividef(1.0f, __fmaf_rn(-q.s, eta, 1.0f)) : 1.0f;
+  float pR = __fmul_rn(__fmul_rn(q.K0, eta), __fmul_rn(id, id));
+  float eR = __fmaf_rn(__fmul_rn(pR, eta), q.inv_2rho0, q.e0), dpR, deR;
+  if (!comp && !(eta >= q.eta_min)) mg_ref<float>(q, eta, pR, dpR, eR, deR);
+  p = __fmaf_rn(q.rg, __fsub_rn(e, eR), pR);
+  return eta < q.eta_max;
+}
+
+// The same in FP64 (fused operations written out: the same bits in every kernel).
+__device__ __forceinline__ bool mg_p(const EosP<double>& q, double inv_rho, double e, double& p) {
+  const double eta = fma(-q.rho0, inv_rho, 1.0);
+  const bool comp = gt0(eta);
+  const double d = fma(comp ? -q.s : 0.0, eta, 1.0);
+  if (!nr_range_pos(d)) return false;  // eta >= 1/s
+  const double id = rcp_nr_in_range(d);
+  double pR = __dmul_rn(__dmul_rn(q.K0, eta), __dmul_rn(id, id));
+  double eR = fma(__dmul_rn(pR, eta), q.inv_2rho0, q.e0), dpR, deR;
+  if (!comp && eta < q.eta_min) mg_ref<double>(q, eta, pR, dpR, eR, deR);
+  p = fma(q.rg, __dsub_rn(e, eR), pR);
+  return true;
+}
+
 // p(rho, e) given 1/rho; false if the state is outside the EOS domain.
 template <typename R, bool EXT = false, int T = -1>
 __device__ __forceinline__ bool eos_p(const EosP<R>& q, R rho, R inv_rho, R e, R& p) {
   if (eos_is<T>(q, M2C_EOS_SG)) {
-    p = q.gm1 * rho * e - q.gpc;
+    if constexpr (sizeof(R) == 8) p = fma(__dmul_rn(q.gm1, rho), e, -q.gpc);
+    else p = q.gm1 * rho * e - q.gpc;
     return true;
   }
   if constexpr (EXT) {
@@ -480,12 +510,8 @@ __device__ __forceinline__ bool eos_p(const EosP<R>& q, R rho, R inv_rho, R e, R
       return true;
     }
   }
-  R eta = (R)1 - q.rho0 * inv_rho;
-  if (!(eta < q.eta_max)) return false;
-  R pR, dpR, eR, deR;
-  mg_ref(q, eta, pR, dpR, eR, deR);
-  p = pR + q.rg * (e - eR);
-  return true;
+  if constexpr (sizeof(R) == 4) return mg_p_f(q, inv_rho, e, p);
+  else return mg_p(q, inv_rho, e, p);
 }
 
 // MG in FP64, e and c^2 from one reciprocal beside 1/rho: with d = 1 - s eta in
@@ -497,9 +523,9 @@ __device__ __forceinline__ bool mg_e_c2(const EosP<double>& q, double inv_rho, d
   const bool comp = gt0(eta);
   const double d = fma(comp ? -q.s : 0.0, eta, 1.0);
   if (!nr_range_pos(d)) return false;  // eta >= 1/s
-  const double id = rcp_nr_in_range(d), w = id * id;
-  double pR = q.K0 * eta * w, a = fma(eta, q.inv_2rho0, -q.inv_rg);
-  double A = fma(fma(comp ? q.sG : -q.G0, eta, 1.0) * (w * id), q.rK, q.rg * p);
+  const double id = rcp_nr_in_range(d), w = __dmul_rn(id, id);
+  double pR = __dmul_rn(__dmul_rn(q.K0, eta), w), a = fma(eta, q.inv_2rho0, -q.inv_rg);
+  double A = fma(__dmul_rn(fma(comp ? q.sG : -q.G0, eta, 1.0), __dmul_rn(w, id)), q.rK, __dmul_rn(q.rg, p));
   double eb = fma(p, q.inv_rg, q.e0);
   if (!comp && eta < q.eta_min) {  // below the tension cutoff the reference pressure is constant
     pR = q.pmin;
@@ -508,8 +534,26 @@ __device__ __forceinline__ bool mg_e_c2(const EosP<double>& q, double inv_rho, d
     eb += q.K0 * q.eta_min * q.eta_min * q.inv_2rho0 + q.pmin / q.rho0 * (eta - q.eta_min);
   }
   e = fma(pR, a, eb);
-  c2 = A * (inv_rho * inv_rho);
+  c2 = __dmul_rn(A, __dmul_rn(inv_rho, inv_rho));
   return true;
+}
+
+// The same in FP32 for the mixed path's face states, without a branch between
+// compression and tension, every rounding written out (those of mg_ref and the
+// general form below).
+__device__ __forceinline__ bool mg_e_c2_f(const EosP<float>& q, float inv_rho, float p, float& e, float& c2) {
+  const float eta = __fmaf_rn(-q.rho0, inv_rho, 1.0f);
+  const bool comp = eta > 0.0f;
+  const float k = __fmul_rn(q.K0, eta);
+  const float id = comp ? __fdividef(1.0f, __fmaf_rn(-q.s, eta, 1.0f)) : 1.0f, id2 = __fmul_rn(id, id);
+  float pR = __fmul_rn(k, id2);
+  float dpR = __fmul_rn(__fmul_rn(__fmul_rn(q.K0, __fmaf_rn(comp ? q.s : 0.0f, eta, 1.0f)), id2), id);
+  float eR = __fmaf_rn(__fmul_rn(pR, eta), q.inv_2rho0, q.e0);
+  float deR = comp ? __fmul_rn(__fmaf_rn(dpR, eta, pR), q.inv_2rho0) : __fmul_rn(k, __fmul_rn(2.0f, q.inv_2rho0));
+  if (!comp && !(eta >= q.eta_min)) mg_ref<float>(q, eta, pR, dpR, eR, deR);
+  e = __fmaf_rn(__fsub_rn(p, pR), q.inv_rg, eR);
+  c2 = __fmul_rn(__fmaf_rn(p, q.rg, __fmul_rn(__fmaf_rn(-q.rg, deR, dpR), q.rho0)), __fmul_rn(inv_rho, inv_rho));
+  return eta < q.eta_max;
 }
 
 // e(rho, p) and c^2(rho, p) together (App. B.3 and App. C.2: c^2 = dp/drho|_e + p/rho^2 dp/de|_rho).
@@ -520,11 +564,12 @@ __device__ __forceinline__ bool eos_e_c2(const EosP<R>& q, R rho, R inv_rho, R p
   if (eos_is<T>(q, M2C_EOS_SG)) {
     if constexpr (sizeof(R) == 8) {
       e = (p + q.gpc) * (q.inv_gm1 * inv_rho);
-      c2 = fma(q.g, p, q.gpc) * inv_rho;
+      c2 = __dmul_rn(fma(q.g, p, q.gpc), inv_rho);
     } else {
       R pb = p + q.pc;
-      e = (p + q.gpc) * q.inv_gm1 * inv_rho;
-      c2 = q.g * pb * inv_rho;
+      // products rounded, not contracted into the sums they enter
+      e = __fmul_rn((p + q.gpc) * q.inv_gm1, inv_rho);
+      c2 = __fmul_rn(q.g * pb, inv_rho);
     }
   } else if (EXT && q.type == M2C_EOS_NASG) {
     // e = e_c + (p + g pc)(1 - rho b)/((g - 1) rho), c^2 = g (p + pc)/(rho (1 - rho b))
@@ -541,13 +586,7 @@ __device__ __forceinline__ bool eos_e_c2(const EosP<R>& q, R rho, R inv_rho, R p
   } else if constexpr (sizeof(R) == 8) {
     if (!mg_e_c2(q, inv_rho, p, e, c2)) return false;
   } else {
-    R eta = (R)1 - q.rho0 * inv_rho;
-    if (!(eta < q.eta_max)) return false;
-    R pR, dpR, eR, deR;
-    mg_ref(q, eta, pR, dpR, eR, deR);
-    e = eR + (p - pR) * q.inv_rg;
-    R ir2 = inv_rho * inv_rho;
-    c2 = ((dpR - q.rg * deR) * q.rho0 + p * q.rg) * ir2;
+    if (!mg_e_c2_f(q, inv_rho, p, e, c2)) return false;
   }
   if constexpr (sizeof(R) == 8) return gt0(c2) && hi_of(c2) < 0x7ff00000u;
   else return c2 > (R)0 && c2 < (R)INFINITY;
@@ -568,8 +607,8 @@ __device__ __forceinline__ R va_slope(R a, R b) {
     const double num = ab * (a + b), den = a * a + b * b;
     return nr_range(den) ? num * rcp_nr_in_range(den) : div_ieee(num, den);
   } else {
-    if (!(ab > (R)0)) return (R)0;
-    return rdiv<R>(ab * (a + b), a * a + b * b);
+    const float s = __fdividef(__fmul_rn(ab, a + b), __fmaf_rn(a, a, __fmul_rn(b, b)));
+    return ab > 0.0f ? s : 0.0f;
   }
 }
 
@@ -642,40 +681,44 @@ __device__ __forceinline__ void hllc64(const FaceState<double>& L, const FaceSta
   F[4] = Ss * fma(fma(aK, K.E, fma(ps, Ss, -K.p * uK)), iS, ps);
 }
 
+// FP32 (mixed path): the formulas as printed, without branches (the sides and the
+// supersonic cases selected), every rounding written out.
+template <int D>
+__device__ __forceinline__ void hllc32(const FaceState<float>& L, const FaceState<float>& Rt, float F[5]) {
+  const float uL = comp<D>(L), uR = comp<D>(Rt);
+  const float SL = fminf(__fsub_rn(uL, L.c), __fsub_rn(uR, Rt.c));
+  const float SR = fmaxf(__fadd_rn(uL, L.c), __fadd_rn(uR, Rt.c));
+  const float aL = __fmul_rn(L.rho, __fsub_rn(SL, uL)), aR = __fmul_rn(Rt.rho, __fsub_rn(SR, uR));
+  const float Ss = __fdividef(__fmaf_rn(-uR, aR, __fmaf_rn(uL, aL, __fsub_rn(Rt.p, L.p))), __fsub_rn(aL, aR));
+  const bool superL = 0.0f <= SL, left = superL || 0.0f <= Ss;
+  const bool star = !superL && (left || 0.0f <= SR);
+  const float rho = left ? L.rho : Rt.rho, u = left ? L.u : Rt.u, v = left ? L.v : Rt.v, w = left ? L.w : Rt.w;
+  const float p = left ? L.p : Rt.p, E = left ? L.E : Rt.E;
+  const float un = left ? uL : uR, SK = left ? SL : SR, aK = left ? aL : aR;
+  const float m = __fmul_rn(rho, un), rE = __fmul_rn(rho, E);
+  const float fac = __fdividef(aK, __fsub_rn(SK, Ss));
+  const float Es = __fmaf_rn(__fsub_rn(Ss, un), Ss + __fdividef(p, aK), E);  // (the sum may take the quotient's product)
+  // S_K (W*_K - W_K)
+  const float V[3] = {u, v, w};
+  F[0] = star ? __fmaf_rn(SK, __fsub_rn(fac, rho), m) : m;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (a == D) {
+      const float f = __fmaf_rn(m, V[a], p);
+      F[1 + a] = star ? __fmaf_rn(SK, __fmaf_rn(fac, Ss, -m), f) : f;
+    } else {
+      const float g = __fmul_rn(SK, __fmaf_rn(fac, V[a], -__fmul_rn(rho, V[a])));
+      F[1 + a] = star ? __fmaf_rn(m, V[a], g) : __fmul_rn(m, V[a]);
+    }
+  }
+  F[4] = star ? __fmaf_rn(__fadd_rn(rE, p), un, __fmul_rn(SK, __fmaf_rn(fac, Es, -rE)))
+              : __fmul_rn(__fmaf_rn(rho, E, p), un);
+}
+
 template <int D, typename R>
 __device__ __forceinline__ void hllc(const FaceState<R>& L, const FaceState<R>& Rt, R F[5]) {
-  if constexpr (sizeof(R) == 8) {
-    hllc64<D>(L, Rt, F);
-    return;
-  }
-  const R uL = comp<D>(L), uR = comp<D>(Rt);
-  const R SL = fmin(uL - L.c, uR - Rt.c);
-  const R SR = fmax(uL + L.c, uR + Rt.c);
-  const R aL = L.rho * (SL - uL), aR = Rt.rho * (SR - uR);
-  const R Ss = rdiv<R>(Rt.p - L.p + uL * aL - uR * aR, aL - aR);
-  if ((R)0 <= SL) {
-    phys_flux<D>(L, F);
-    return;
-  }
-  bool left;
-  if ((R)0 <= Ss) left = true;
-  else if ((R)0 <= SR) left = false;
-  else {
-    phys_flux<D>(Rt, F);
-    return;
-  }
-  const FaceState<R>& K = left ? L : Rt;
-  const R SK = left ? SL : SR;
-  const R uK = left ? uL : uR;
-  const R aK = left ? aL : aR;
-  phys_flux<D>(K, F);
-  const R fac = rdiv<R>(aK, SK - Ss);
-  const R Es = K.E + (Ss - uK) * (Ss + rdiv<R>(K.p, aK));
-  R ws[5] = {fac, fac * K.u, fac * K.v, fac * K.w, fac * Es};
-  ws[1 + D] = fac * Ss;
-  const R wk[5] = {K.rho, K.rho * K.u, K.rho * K.v, K.rho * K.w, K.rho * K.E};
-#pragma unroll
-  for (int v = 0; v < 5; ++v) F[v] = F[v] + SK * (ws[v] - wk[v]);
+  if constexpr (sizeof(R) == 8) hllc64<D>(L, Rt, F);
+  else hllc32<D>(L, Rt, F);
 }
 
 // Local Lax-Friedrichs flux (App. C.1, Eq. Lax-Friedrichs):

@@ -783,14 +783,15 @@ m2c_status push_grid(m2c_ctx* c) {
 // spread a small grid over the SMs and even out tiles of unequal cost (a
 // locally uniform plane is cheaper). Estimated launch time in plane times of one
 // resident block: below one tile per slot the tiles run side by side, the most
-// loaded SM sets the time; above, the tiles' planes over the slots plus half a
-// tile of tail. slots = resident blocks x SMs; t1 and tR are the times of a
-// plane with one and with all `blocks` of them on the SM: a plane takes 14 us
-// alone and 17-20 us beside three others in the mixed kernel (8 rows; latency
+// loaded SM sets the time; above, the tiles' planes over the slots plus three
+// quarters of a tile of tail. slots = resident blocks x SMs; t1 and tR are the
+// times of a plane with one and with all `blocks` of them on the SM: a plane takes
+// 9 us alone and 13.5 us beside another in the mixed kernel (8 rows; latency
 // bound), and as long as the FP64 pipe needs in the FP64 kernel. Measured per
-// launch with the former fixed 16-plane chunks and now: 48^3 mixed 242 -> 38 us,
-// 131x67x45 mixed 381 -> 120, 112^3 mixed 281 -> 201, 192^3 mixed 1184 -> 1021
-// (16 rows), 128x4x4 FP64 207 -> 55, 128^3 FP64 2795 -> 2664.
+// launch with fixed 16-plane chunks, and with this rule on the same kernel:
+// 48^3 mixed 242 -> 38 us, 131x67x45 mixed 381 -> 120, 112^3 mixed 281 -> 201,
+// 128x4x4 FP64 207 -> 55, 128^3 FP64 2795 -> 2664 (the present kernel: 48^3
+// 34.5, 131x67x45 103, 128x4x4 40, 128^3 FP64 1277).
 struct TileShape {
   int rows, blocks;
   double t1, tR;
@@ -830,8 +831,8 @@ int choose_tz(const Grid* const* g, int n, const TileShape& s, double* best_out 
 
 TileShape tile_shape(int prec, int rows) {
   if (prec == M2C_FP64) return rows == 4 ? TileShape{4, 2, 0.75, 1.05} : TileShape{8, 1, 1.0, 1.0};
-  if (rows == 16) return TileShape{16, 2, 15.5, 17.5};
-  return rows == 4 ? TileShape{4, 6, 14.0, 18.0} : TileShape{8, 4, 14.0, 19.0};
+  if (rows == 16) return TileShape{16, 1, 15.0, 15.0};
+  return rows == 4 ? TileShape{4, 4, 9.0, 13.0} : TileShape{8, 2, 9.0, 13.5};
 }
 
 int default_tz(const Grid& g, int ty) {
@@ -839,16 +840,16 @@ int default_tz(const Grid& g, int ty) {
   return choose_tz(one, 1, tile_shape(g.prec, ty));
 }
 
-// Tile rows: 8, or the other shape of the precision when its estimate is lower
-// (16 rows on the mixed path for large grids, whose halo rows are fewer: 1947 against 2125 us per
-// launch at 256^3; 4 rows on the FP64 path for grids with too few tiles).
+// Tile rows: 8 (16 rows on the mixed path hold as many threads on an SM and, as one
+// block, wait for each other at every barrier); 4 on the FP64 path for grids with
+// too few tiles of 8.
 int default_rows(const Grid& g) {
+  if (g.prec == M2C_MIXED) return 8;
   const Grid* one[1] = {&g};
-  double e8, eo;
-  const int other = g.prec == M2C_MIXED ? 16 : 4;
+  double e8, e4;
   choose_tz(one, 1, tile_shape(g.prec, 8), &e8);
-  choose_tz(one, 1, tile_shape(g.prec, other), &eo);
-  return eo < e8 ? other : 8;
+  choose_tz(one, 1, tile_shape(g.prec, 4), &e4);
+  return e4 < e8 ? 4 : 8;
 }
 
 // Event pairs recorded around launches while profiling, tagged with the kernel kind.
@@ -1326,6 +1327,7 @@ m2c_status m2c_step(m2c_ctx* c, int nsteps) {
     LaunchPlan lp;
     lp.ty = c->ty;
     lp.mats = material_pair(c->host);
+    lp.one = &c->host;
     cudaError_t e = enqueue_step(c->dev_grid, c->dev_tiles, 1, ntiles_of(c->host), c->host.prec, lp, re,
                                  c->reinit_iters, c->host.N, c->stream, c->profiling ? &pe : nullptr, c->host.rk,
                                  c->host.general != 0, c->host.band_gamma > 0.0);
@@ -1499,6 +1501,7 @@ m2c_status m2c_residual(m2c_ctx* c, double* R, double* L) {
   LaunchPlan lp;
   lp.ty = c->ty;
   lp.mats = material_pair(c->host);
+  lp.one = &c->host;
   cudaError_t e = launch_stage(c->host.prec, c->dev_grid, c->dev_tiles, 1, ntiles_of(c->host), kResidual, lp,
                                c->stream, c->host.general != 0);
   if (e == cudaSuccess) {
@@ -1784,6 +1787,7 @@ m2c_status m2c_residual_noalloc(int nx, int ny, int nz, double h, const int bc[6
   LaunchPlan lp;
   lp.ty = ty;
   lp.mats = material_pair(g);
+  lp.one = &g;
   if (e == cudaSuccess) e = launch_stage(precision, dg, dt, 1, tiles[1], kResidual, lp, s);
   if (e == cudaSuccess) {
     const dim3 lg((unsigned)(2 * sm_count()), 1);

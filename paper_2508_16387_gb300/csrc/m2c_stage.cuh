@@ -14,23 +14,30 @@ namespace m2c {
 // Bulk stage kernel
 // ---------------------------------------------------------------------------
 
-// The level set and material planes are double-buffered where shared memory
-// allows (16-row FP32 tiles at two blocks per SM, FP64 tiles at one): a plane's
-// update reads them while the next plane's loads already write the other
-// buffer, which saves one block barrier per plane. The 8-row FP32 tiles (four
-// blocks per SM) keep one buffer and the barrier.
+// Shared memory of a tile: the plane being worked on and the next one (primitive
+// fields, level set, material ids, with a two-cell halo); what a row hands to the
+// row on its minus side (ym, the MUSCL states on the minus y faces of rows 0 ..
+// TY) and on its plus side (yf, the fluxes through the plus y faces; row 0 is the
+// tile's minus face); the states on both sides of the tile's two x faces (xe: cells
+// -1, 0, 31, 32 of every row) and the fluxes through them (xf); the plus states of
+// row -1 (yp); per thread the plus z state of
+// its next cell (qz) and the last two z fluxes (fz); per row which cells equal
+// those of the next row (ey), and whether its end faces count (ex).
 template <typename R, int TY>
 struct StageSmem {
-  static constexpr int TX = 32, HX = TX + 4, HY = TY + 4;
-  static constexpr int NB = (TY >= 16 || sizeof(R) == 8) ? 2 : 1;
+  static constexpr int TX = 32, HX = TX + 4, HY = TY + 4, PL = HX * HY, NT = TX * TY;
   static constexpr size_t q_off = 0;
-  static constexpr size_t phi_off = q_off + sizeof(R) * 5 * HY * HX;
-  static constexpr size_t xs_off = phi_off + sizeof(R) * NB * HY * HX;
-  static constexpr size_t ys_off = xs_off + sizeof(FaceState<R>) * TY * (TX + 2) * 2;
-  static constexpr size_t fx_off = ys_off + sizeof(FaceState<R>) * (TY + 2) * TX * 2;
-  static constexpr size_t fy_off = fx_off + sizeof(R) * 5 * TY * (TX + 1);
-  static constexpr size_t id_off = fy_off + sizeof(R) * 5 * (TY + 1) * TX;
-  static constexpr size_t bytes = (id_off + NB * HY * HX + 15) / 16 * 16;
+  static constexpr size_t phi_off = q_off + sizeof(R) * 2 * 5 * PL;
+  static constexpr size_t ym_off = phi_off + sizeof(R) * 2 * PL;
+  static constexpr size_t yf_off = ym_off + sizeof(R) * 7 * (TY + 1) * TX;
+  static constexpr size_t qz_off = yf_off + sizeof(R) * 5 * (TY + 1) * TX;
+  static constexpr size_t fz_off = qz_off + sizeof(R) * 7 * NT;
+  static constexpr size_t xe_off = fz_off + sizeof(R) * 2 * 5 * NT;
+  static constexpr size_t xf_off = xe_off + sizeof(R) * 7 * 4 * TY;
+  static constexpr size_t yp_off = xf_off + sizeof(R) * 5 * 2 * TY;
+  static constexpr size_t ey_off = yp_off + sizeof(R) * 7 * TX;
+  static constexpr size_t id_off = ey_off + sizeof(unsigned) * (2 * TY + 4);
+  static constexpr size_t bytes = (id_off + 2 * PL + 15) / 16 * 16;
 };
 
 // Compile-time integer for the material dispatch below (usable in device code).
@@ -57,16 +64,82 @@ __device__ __forceinline__ void by_material(int m, F&& f) {
   }
 }
 
-// FP64 tiles run one block per SM (FP64-pipe bound); the FP32 tiles of the
-// mixed path are latency bound and are compiled for 1024 resident threads per
-// SM (64 registers a thread): four 256-thread blocks of 8-row tiles (55 KB of
-// shared memory each) or two 512-thread blocks of 16-row tiles.
+// Face states of a cell of material ic along one axis (cell_faces). For FP32 and a
+// fixed pair of types the slopes, the face values and everything but e and c^2 are
+// one code for both materials (a warp across the interface takes only the equation
+// of state twice), without branches but for states that are not admissible; a zero
+// slope gives the cell state itself.
+template <bool GEN, int MT, typename R, typename EA>
+__device__ __forceinline__ void material_faces(EA&& eos, int ic, const R Pm[5], const R P[5], const R Pp[5], bool same,
+                                               FaceState<R>& QM, FaceState<R>& QP, bool& bad, int lim, R alpha) {
+  if constexpr (sizeof(R) == 4 && !GEN && MT >= 0) {
+    float a[5], b[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const float s = va_slope<float>(P[v] - Pm[v], Pp[v] - P[v]), h = same ? s : 0.0f;
+      a[v] = __fmaf_rn(-0.5f, h, P[v]);
+      b[v] = __fmaf_rn(0.5f, h, P[v]);
+    }
+    const float ia = rrcp<float>(a[0]), ib = rrcp<float>(b[0]);
+    float ea, ca, eb, cb;
+    bool oka, okb;
+    by_material<MT>(ic, [&](auto T, auto m) {
+      oka = face_eos_f<decltype(T)::value>(eos(m), a[0], ia, a[4], ea, ca);
+      okb = face_eos_f<decltype(T)::value>(eos(m), b[0], ib, b[4], eb, cb);
+    });
+    if (!(oka && okb)) {
+      // first order (Reading R12)
+      by_material<MT>(ic, [&](auto T, auto m) {
+        oka = face_eos_f<decltype(T)::value>(eos(m), P[0], rrcp<float>(P[0]), P[4], ea, ca);
+      });
+      if (!oka) bad = true;
+      okb = oka;
+      eb = ea;
+      cb = ca;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) a[v] = b[v] = P[v];
+    }
+    finish_face_f(a, ea, ca, oka, QM);
+    finish_face_f(b, eb, cb, okb, QP);
+  } else {
+    by_material<MT>(ic, [&](auto T, auto m) {
+      cell_faces<R, GEN, decltype(T)::value>(eos(m), Pm, P, Pp, same, QM, QP, bad, lim, alpha);
+    });
+  }
+}
+
+// A tile is 32 x TY columns marching along z, one warp per row of 32 cells, one
+// thread per column. Per plane and thread: the face states along z (from a register
+// window), x and y (from the shared plane) of its own cell, the fluxes through its
+// own plus faces with the neighbour's minus state (by shuffle along x, through
+// shared memory along y), the residual and the update. The cells and faces just
+// outside the tile that its fluxes need (columns -1 and 32, rows -1 and TY) are
+// taken by three warps on top of their own row, the halo loads by others. The
+// face states of all of them are one loop, so that the reconstruction and the
+// equation of state are one piece of code (six copies of it doubled the stalls for
+// instructions). Two block barriers per plane: after the minus states, and after
+// the y fluxes; plane k+1 is staged during plane k, so that the update of a plane
+// and the loads and face states of the next run without a barrier between them.
 //
-// Every thread's share of the plane work (halo cell, face-state items, flux
-// items) and its shared-memory addresses are fixed for the whole launch; only
-// the plane index changes along the march. The halo slots are computed once,
-// the face-state and flux items are recomputed from the thread index where
-// they are used (cheaper than holding them in registers across the march).
+// Uniform rows. Where a cell and its two neighbours along an axis hold the same
+// primitive state and material, its slopes and those of the neighbours towards it
+// vanish, both fluxes of the axis are the flux of that one state, and their
+// difference is exactly zero. A warp whose 32 cells and their neighbours are so
+// along an axis leaves out the axis' face states and fluxes (fluid at rest ahead
+// of a shock, the uniform state behind it, the inside of a bubble: most of the
+// domain until the waves have crossed it); one uniform along all three copies the
+// state. The results are the same bits.
+//
+// What bounds it: FP32 tiles the instruction issue and the latency of each warp's
+// chain (about 820 instructions a cell and stage without any face state, 1700 in an
+// early shock-bubble), compiled for 512 resident threads per SM (128 registers, no
+// spills; with 1024 threads at 64 registers the spills went to L2, the shared memory
+// leaving little L1, and took as long); FP64 tiles the FP64 pipe. Against face states
+// and fluxes as items distributed over the threads (2.2 and 2.1 a thread, all states
+// and fluxes through shared memory, three barriers, no uniform rows), per launch:
+// 256^3 mixed 1947 -> 1617 us, 192^3 with the shock in the bubble 1028 -> 927,
+// 131x67x45 120 -> 103, 48^3 38 -> 34.5; FP64 128^3 2064 -> 1277, 75x51x67 with
+// mirrors 507 -> 380.
 //
 // GEN = false is the default scheme (TVD RK2, modified van Albada, HLLC); GEN =
 // true is the general instantiation, which takes the grid's scheme options at
@@ -74,96 +147,78 @@ __device__ __forceinline__ void by_material(int m, F&& f) {
 // MT >= 0 fixes the EOS types of the two materials (SG or MG, MT = T0 + 4 T1)
 // for launches whose grids all have that pair, which removes the type dispatch
 // from every EOS evaluation; MT = -1 reads the types at run time.
-template <typename R, int TY, bool GEN, int MT = -1>
-__global__ void __launch_bounds__(32 * TY, (sizeof(R) == 8 ? 1 : 1024 / (32 * TY)))
-k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin, int ngrid, long long ntiles, int mode,
-        int sched, unsigned long long* __restrict__ tile_counter) {
+//
+// ONE (mixed path, default scheme): the launch's only grid comes as a kernel
+// parameter, so that its pointers, sizes and EOS constants are constant-bank operands
+// instead of loads from shared memory and registers; else the descriptor of the
+// tile's grid is copied to shared memory.
+template <bool ONE>
+struct StageArg {
+  Grid grid;
+};
+template <>
+struct StageArg<false> {};
+
+template <typename R, int TY, bool GEN, int MT, bool ONE>
+__global__ void __launch_bounds__(32 * TY, (sizeof(R) == 8 ? 1 : 512 / (32 * TY)))
+k_stage(const __grid_constant__ StageArg<ONE> arg, const Grid* __restrict__ grids,
+        const long long* __restrict__ tile_begin, int ngrid, long long ntiles, int mode, int sched,
+        unsigned long long* __restrict__ tile_counter) {
   constexpr int TX = 32, NT = TX * TY, HX = TX + 4, HY = TY + 4, PL = HY * HX;
-  constexpr int NXS = (TX + 2) * TY, NYS = TX * (TY + 2), NS = NXS + NYS;  // face-state items
-  constexpr int NXF = (TX + 1) * TY, NYF = TX * (TY + 1), NF = NXF + NYF;  // flux items
-  constexpr int NHALO = 4 * (TX + TY);
-  constexpr int SI = (NS + NT - 1) / NT, FI = (NF + NT - 1) / NT;
-  constexpr int SFX = TY * (TX + 1), SFY = (TY + 1) * TX;                   // flux array strides
+  // halo cells of a plane: four columns of TY (padded to whole warps), then four rows of 32
+  constexpr int NHX = (4 * TY + 31) / 32 * 32, NHALO = NHX + 4 * TX;
+  constexpr int HI = (NHALO + NT - 1) / NT;
+  // warps with work outside the tile: the cells of columns -1 and 32, of row -1, of row TY
+  constexpr int kWarpX = TY - 3, kWarpY0 = TY - 2, kWarpY1 = TY - 1;
+  static_assert(TY >= 4 && 2 * TY <= 32, "columns -1 and 32 of a tile are the lanes of one warp");
   using SM = StageSmem<R, TY>;
+  constexpr int SYM = (TY + 1) * TX, SXE = 4 * TY;  // strides of the state and flux components
   extern __shared__ __align__(16) unsigned char smem[];
-  R* s_q = reinterpret_cast<R*>(smem + SM::q_off);                         // [5][HY][HX]
-  R* const s_phi0 = reinterpret_cast<R*>(smem + SM::phi_off);               // [NB][HY][HX]
-  FaceState<R>* s_st = reinterpret_cast<FaceState<R>*>(smem + SM::xs_off);  // x: [TY][TX+2][2], then y: [TY+2][TX][2]
-  R* s_fx = reinterpret_cast<R*>(smem + SM::fx_off);                       // [5][TY][TX+1]
-  R* s_fy = reinterpret_cast<R*>(smem + SM::fy_off);                       // [5][TY+1][TX]
-  uint8_t* const s_id0 = smem + SM::id_off;                                // [NB][HY][HX]
-  // the descriptor of the tile's grid, copied to shared memory for each tile
+  R* const s_q = reinterpret_cast<R*>(smem + SM::q_off);      // [2][5][HY][HX]
+  R* const s_phi = reinterpret_cast<R*>(smem + SM::phi_off);  // [2][HY][HX]
+  R* const s_ym = reinterpret_cast<R*>(smem + SM::ym_off);    // [7][TY+1][32]
+  R* const s_yf = reinterpret_cast<R*>(smem + SM::yf_off);    // [5][TY+1][32]
+  R* const s_qz = reinterpret_cast<R*>(smem + SM::qz_off);    // [7][NT]
+  R* const s_fz = reinterpret_cast<R*>(smem + SM::fz_off);    // [2][5][NT]
+  R* const s_xe = reinterpret_cast<R*>(smem + SM::xe_off);    // [7][4][TY]: plus state of cell -1, minus of 0, plus of 31, minus of 32
+  R* const s_xf = reinterpret_cast<R*>(smem + SM::xf_off);    // [5][2][TY]
+  R* const s_yp = reinterpret_cast<R*>(smem + SM::yp_off);    // [7][32]
+  unsigned* const s_ey = reinterpret_cast<unsigned*>(smem + SM::ey_off);  // [TY+3], rows -2 .. TY
+  unsigned* const s_ex = s_ey + TY + 3;                                   // [TY]
+  uint8_t* const s_id = smem + SM::id_off;                    // [2][HY][HX]
+  // the descriptor of the tile's grid: the parameter, or copied to shared memory for each tile
   // (its fields and EOS parameters are read all through the plane loop)
-  __shared__ __align__(16) Grid s_G;
+  constexpr size_t kGridBytes = ONE ? 16 : sizeof(Grid);
+  __shared__ __align__(16) unsigned char s_grid[kGridBytes];
   static_assert(sizeof(Grid) % 8 == 0, "grid descriptor copy");
-  const EosP<R>* s_eos;
-  if constexpr (sizeof(R) == 8) s_eos = s_G.eos;
-  else s_eos = s_G.eosf;
-  const EosDev* s_eosd = s_G.eos;
+  const Grid* Gp;
+  if constexpr (ONE) Gp = &arg.grid;
+  else Gp = reinterpret_cast<const Grid*>(s_grid);
+  const Grid& G = *Gp;
+  auto eos = [&](auto m) -> const EosP<R>& {
+    if constexpr (sizeof(R) == 8) return G.eos[m];
+    else return G.eosf[m];
+  };
+  auto eosd = [&](auto m) -> const EosDev& { return G.eos[m]; };
   __shared__ double s_dt;
   __shared__ double s_red[32];
   __shared__ long long s_tile;
 
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const unsigned lane = tid & 31, lt = (1u << lane) - 1u;
-
-  // The thread's share of the plane work is recomputed from the thread index
-  // where it is used (a volatile read of %tid.x keeps the compiler from
-  // holding the items in registers across the plane loop).
-  auto tid_now = []() {
-    unsigned t;
-    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
-    return (int)t;
-  };
-  // face-state item s, packed: centre in the plane buffer (bits 0-9), stencil along y (bit 10); -1: none
-  auto st_item = [&](int s) {
-    const int i = tid_now() + s * NT;
-    if (i < NXS) return (i / (TX + 2) + 2) * HX + i % (TX + 2) + 1;
-    if (i < NS) {
-      const int j = i - NXS;
-      return ((j / TX + 1) * HX + j % TX + 2) | (1 << 10);
-    }
-    return -1;
-  };
-  // flux item s, packed in two words: left face state (bits 0-15) and direction y (bit 30),
-  // -1: none; id position of the left cell (bits 0-15) and output offset (bits 16-31)
-  auto flux_item = [&](int s, int& b) {
-    const int i = tid_now() + s * NT;
-    if (i < NXF) {
-      const int f = i % (TX + 1), row = i / (TX + 1);
-      b = ((row + 2) * HX + f + 1) | ((row * (TX + 1) + f) << 16);
-      return 2 * (row * (TX + 2) + f) + 1;
-    }
-    if (i < NF) {
-      const int j = i - NXF;
-      const int x = j % TX, f = j / TX;
-      b = ((f + 1) * HX + x + 2) | ((f * TX + x) << 16);
-      return (2 * NXS + 2 * (f * TX + x) + 1) | (1 << 30);
-    }
-    b = 0;
-    return -1;
-  };
-  static_assert(2 * NS < 65536 && PL < 1024 && SFX < 32768 && SFY < 32768, "packed item fields");
-  // halo cells of the plane buffer loaded by this thread (two-cell ring without corners):
-  // smem slot, or -1
-  constexpr int HI = (NHALO + NT - 1) / NT;
-  int h_hx[HI], h_hy[HI];
-#pragma unroll
-  for (int s = 0; s < HI; ++s) {
-    const int h = tid + s * NT;
-    h_hx[s] = -1;
-    h_hy[s] = 0;
+  // halo cell s of a plane loaded by this thread (two-cell ring without corners): its slot, -1: none
+  auto halo_slot = [&](int s) {
+    const int h = tid + s * NT, h2 = h - NHX;
     if (h < 4 * TY) {
       const int c4 = h / TY;
-      h_hx[s] = c4 < 2 ? c4 : TX + c4;
-      h_hy[s] = h % TY + 2;
-    } else if (h < NHALO) {
-      const int h2 = h - 4 * TY;
-      const int c4 = h2 / TX;
-      h_hy[s] = c4 < 2 ? c4 : TY + c4;
-      h_hx[s] = h2 % TX + 2;
+      return (h % TY + 2) * HX + (c4 < 2 ? c4 : TX + c4);
     }
-  }
+    if (h2 >= 0 && h2 < 4 * TX) {
+      const int c4 = h2 / TX;
+      return (c4 < 2 ? c4 : TY + c4) * HX + h2 % TX + 2;
+    }
+    return -1;
+  };
 
   // Tiles of all grids of the launch, taken in order by a fixed stride
   // (sched 0) or from an atomic counter (sched 1).
@@ -177,18 +232,19 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
     tile = blockIdx.x + iter * (long long)gridDim.x;
   }
   if (tile >= ntiles) break;
-  const int gidx = find_grid(tile_begin, ngrid, tile);
-  {
+  long long t = tile;
+  if constexpr (!ONE) {
+    const int gidx = find_grid(tile_begin, ngrid, tile);
     const unsigned long long* src = reinterpret_cast<const unsigned long long*>(grids + gidx);
-    unsigned long long* dst = reinterpret_cast<unsigned long long*>(&s_G);
+    unsigned long long* dst = reinterpret_cast<unsigned long long*>(s_grid);
     for (int i = tid; i < (int)(sizeof(Grid) / 8); i += NT) dst[i] = __ldg(src + i);
+    t -= tile_begin[gidx];
+    __syncthreads();
   }
-  __syncthreads();
-  const Grid& G = s_G;
   const int nx = G.nx, ny = G.ny, nz = G.nz;
-  const long long N = G.N, nxy = (long long)nx * ny;
+  const long long N = G.N;
+  const int nxy = nx * ny;
   const int bcz0 = G.bc[4], bcz1 = G.bc[5];
-  long long t = tile - tile_begin[gidx];
   const int bx = (int)(t % G.tiles_x);
   t /= G.tiles_x;
   const int by = (int)(t % G.tiles_y);
@@ -215,26 +271,21 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
 
   const int gx = x0 + tx, gy = y0 + ty;
   const bool inside = gx < nx && gy < ny;
-  // column bases (x, y mapped once per tile)
-  const long long own_base = (long long)map_index(gy, ny, G.bc[2], G.bc[3]) * nx + map_index(gx, nx, G.bc[0], G.bc[1]);
-  long long halo_base[HI];
-#pragma unroll
-  for (int s = 0; s < HI; ++s)
-    halo_base[s] = h_hx[s] < 0 ? 0
-                               : (long long)map_index(y0 + h_hy[s] - 2, ny, G.bc[2], G.bc[3]) * nx +
-                                     map_index(x0 + h_hx[s] - 2, nx, G.bc[0], G.bc[1]);
+  // column bases (x, y mapped once per tile; a grid has fewer than 2^31 cells)
+  const int own_base = map_index(gy, ny, G.bc[2], G.bc[3]) * nx + map_index(gx, nx, G.bc[0], G.bc[1]);
+  int halo_base[HI];
   // general kernel: velocity components to negate for a position mirrored across a
   // symmetry side (bit 0: u, bit 1: v, bit 2: w), for the own column and the halo slots
   int own_neg = 0, halo_neg[HI];
+  if constexpr (GEN) own_neg = mirrored(gx, nx, G.bc[0], G.bc[1]) | (mirrored(gy, ny, G.bc[2], G.bc[3]) << 1);
 #pragma unroll
-  for (int s = 0; s < HI; ++s) halo_neg[s] = 0;
-  if constexpr (GEN) {
-    own_neg = mirrored(gx, nx, G.bc[0], G.bc[1]) | (mirrored(gy, ny, G.bc[2], G.bc[3]) << 1);
-#pragma unroll
-    for (int s = 0; s < HI; ++s)
-      if (h_hx[s] >= 0)
-        halo_neg[s] = mirrored(x0 + h_hx[s] - 2, nx, G.bc[0], G.bc[1]) |
-                      (mirrored(y0 + h_hy[s] - 2, ny, G.bc[2], G.bc[3]) << 1);
+  for (int s = 0; s < HI; ++s) {
+    const int slot = halo_slot(s), hx = x0 + slot % HX - 2, hy = y0 + slot / HX - 2;
+    halo_base[s] = slot < 0 ? 0 : map_index(hy, ny, G.bc[2], G.bc[3]) * nx + map_index(hx, nx, G.bc[0], G.bc[1]);
+    halo_neg[s] = 0;
+    if constexpr (GEN) {
+      if (slot >= 0) halo_neg[s] = mirrored(hx, nx, G.bc[0], G.bc[1]) | (mirrored(hy, ny, G.bc[2], G.bc[3]) << 1);
+    }
   }
   auto zneg = [&](int k) { return GEN ? (mirrored(k, nz, bcz0, bcz1) << 2) : 0; };
 
@@ -242,19 +293,16 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
   bool bad = false, ovf = false;
   // material at the start of the step and the stage state of cell index c
   // (neg: the velocity components to negate, general kernel only)
-  auto load = [&](long long c, R P[5], R& ph, int& idv, int neg) {
+  auto load = [&](int c, R P[5], R& ph, int& idv, int neg) {
     const double phd = gld(phis + c);
-    if (ids_frozen) {
-      idv = __ldg(idg + c) & 1;
-    } else {
-      idv = lt0(phd) ? 1 : 0;
-    }
+    if (ids_frozen) idv = __ldg(idg + c) & 1;
     const double w0 = gld(Ws + c), w1 = gld(Ws + N + c), w2 = gld(Ws + 2 * N + c), w3 = gld(Ws + 3 * N + c),
                  w4 = gld(Ws + 4 * N + c);
     if constexpr (sizeof(R) == 8) {
       ph = phd;
+      if (!ids_frozen) idv = lt0(phd) ? 1 : 0;
       by_material<MT>(idv, [&](auto T, auto m) {
-        if (!cons_to_prim_v<R, GEN, decltype(T)::value>(s_eos[m], s_eosd[m], w0, w1, w2, w3, w4, P)) bad = true;
+        if (!cons_to_prim_v<R, GEN, decltype(T)::value>(eos(m), eosd(m), w0, w1, w2, w3, w4, P)) bad = true;
       });
     } else {
       // the level set and the state's first four components: one group of conversions
@@ -262,10 +310,15 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
       float y[5];
       d2f_group<5>(x, y);
       ph = y[0];
+      if (!ids_frozen) idv = lt0(phd, y[0]) ? 1 : 0;
+      P[0] = y[1];
+      const float inv = rrcp<float>(y[1]);
+      const double rhoe = prim_velocities_f(inv, y[2], y[3], y[4], w4, P);
+      bool ok;
       by_material<MT>(idv, [&](auto T, auto m) {
-        if (!cons_to_prim_f<GEN, decltype(T)::value>(s_eos[m], s_eosd[m], w0, y[1], y[2], y[3], y[4], w4, P))
-          bad = true;
+        ok = prim_pressure_f<GEN, decltype(T)::value>(eos(m), eosd(m), w0, y[1], inv, rhoe, P[4]);
       });
+      bad = bad || !ok || !gt0(w0, y[1]);
     }
     if constexpr (GEN) {
       if (neg & 1) P[1] = -P[1];
@@ -273,30 +326,94 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
       if (neg & 4) P[3] = -P[3];
     }
   };
-  auto plane = [&](int k) { return (long long)map_index(k, nz, bcz0, bcz1) * nxy; };
+  auto plane = [&](int k) { return map_index(k, nz, bcz0, bcz1) * nxy; };
 
-  // ---- warm-up of the z window: planes k0-2 .. k0+1
-  R Pa[5], P0[5], P1[5], P2[5];
+  // rows of a tile cut by the grid's edge: those inside, and the two beyond it that hold halo
+  // cells (the first one's y states are needed too); the others do nothing
+  const bool row_in = gy < ny, row_y = gy <= ny, row_on = gy <= ny + 1;
+  const int cslot = (ty + 2) * HX + tx + 2;
+  auto put = [&](int b, int slot, const R P[5], R phv, int idv) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) s_q[(b * 5 + v) * PL + slot] = P[v];
+    s_phi[b * PL + slot] = phv;
+    s_id[b * PL + slot] = (uint8_t)idv;
+  };
+  auto put_halo = [&](int b, int k) {
+    const int pk = k * nxy;  // k is inside the grid
+#pragma unroll
+    for (int s = 0; s < HI; ++s) {
+      const int slot = halo_slot(s);
+      if (slot < 0) continue;
+      R Ph[5], phh;
+      int idh;
+      load(pk + halo_base[s], Ph, phh, idh, halo_neg[s]);
+      put(b, slot, Ph, phh, idh);
+    }
+  };
+  // whether the cells at two slots of a shared plane hold the same primitive state (finite) and material
+  auto alike = [](const R* q, const uint8_t* idp, int c0, int c1) {
+    bool f = (idp[c0] == idp[c1]) & is_finite(q[4 * PL + c0]);
+#pragma unroll
+    for (int v = 0; v < 5; ++v) f = f & same_bits(q[v * PL + c0], q[v * PL + c1]);
+    return f;
+  };
+  // Uniformity of a staged plane, known to all warps after the next barrier: bit x of mx, cells x and
+  // x + 1 of the own row alike; mx_ends, those at the row's ends too (-2 and -1, -1 and 0, 32 and 33;
+  // only looked at where all of mx are); s_ey, the cells of a row and of the next one.
+  unsigned mx = 0;
+  bool mx_ends = false;
+  auto look_at = [&](int b) {
+    const R* const q = s_q + b * 5 * PL;
+    const uint8_t* const idp = s_id + b * PL;
+    if (row_in) {
+      mx = __ballot_sync(0xffffffffu, alike(q, idp, cslot, cslot + 1));
+      mx_ends = false;
+      if (mx == 0xffffffffu) {
+        const int c0 = (ty + 2) * HX + (tx < 2 ? tx : (tx == 2 ? TX + 2 : 2));
+        mx_ends = __all_sync(0xffffffffu, alike(q, idp, c0, c0 + 1));
+      }
+      if (tx == 0) s_ex[ty] = mx_ends;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, alike(q, idp, cslot, cslot + HX));
+    if (tx == 0) s_ey[ty + 2] = m;
+    if (ty >= kWarpX) {  // rows -2, -1 and TY
+      const int row = ty == kWarpX ? -2 : (ty == kWarpY0 ? -1 : TY);
+      const int c0 = (row + 2) * HX + tx + 2;
+      const unsigned mr = __ballot_sync(0xffffffffu, alike(q, idp, c0, c0 + HX));
+      if (tx == 0) s_ey[row + 2] = mr;
+    }
+  };
+  auto put_state = [](R* o, int stride, const FaceState<R>& Q) {
+    o[0] = Q.rho;
+    o[stride] = Q.u;
+    o[2 * stride] = Q.v;
+    o[3 * stride] = Q.w;
+    o[4 * stride] = Q.p;
+    o[5 * stride] = Q.c;
+    o[6 * stride] = Q.E;
+  };
+  auto get_state = [](const R* o, int stride) {
+    return FaceState<R>{o[0], o[stride], o[2 * stride], o[3 * stride], o[4 * stride], o[5 * stride], o[6 * stride]};
+  };
+
+  // ---- opening of the z window: planes k0-2 .. k0+1, the flux through the tile's lower z face
+  R P1[5], P2[5];
   R ph[5];
-  int ida, idm, id0, id1, id2;
-  FaceState<R> QzP, Qtmp, QzM1, QzP1;
-  R Fzm[5], Fzp[5];
+  int idm, id0, id1, id2;
+  // along z: the cell of plane k is uniform, all of the row's are, qz holds the row's plus states
+  bool flat_z0 = false, rowflat_z0 = false, qz_set = true, alike_z = false;
   {
-    R Pb[5];
-    int idb;
+    R Pb[5], Pa[5], P0[5];
+    FaceState<R> QzP;
+    R Fzm[5];
+    int idb, ida;
     load(plane(k0 - 2) + own_base, Pb, ph[0], idb, own_neg | zneg(k0 - 2));
     load(plane(k0 - 1) + own_base, Pa, ph[1], ida, own_neg | zneg(k0 - 1));
     load(plane(k0) + own_base, P0, ph[2], id0, own_neg);
     load(plane(k0 + 1) + own_base, P1, ph[3], id1, own_neg | zneg(k0 + 1));
-    FaceState<R> QaP, Q0M;
-    by_material<MT>(ida, [&](auto T, auto m) {
-      cell_faces<R, GEN, decltype(T)::value>(s_eos[m], Pb, Pa, P0, idb == ida && id0 == ida, Qtmp, QaP, bad, lim,
-                                              alpha);
-    });
-    by_material<MT>(id0, [&](auto T, auto m) {
-      cell_faces<R, GEN, decltype(T)::value>(s_eos[m], Pa, P0, P1, ida == id0 && id1 == id0, Q0M, QzP, bad, lim,
-                                              alpha);
-    });
+    FaceState<R> Qtmp, QaP, Q0M;
+    material_faces<GEN, MT, R>(eos, ida, Pb, Pa, P0, idb == ida && id0 == ida, Qtmp, QaP, bad, lim, alpha);
+    material_faces<GEN, MT, R>(eos, id0, Pa, P0, P1, ida == id0 && id1 == id0, Q0M, QzP, bad, lim, alpha);
     if (ida == id0) {
       num_flux<2, R, GEN>(QaP, Q0M, Fzm, flx);
     } else {
@@ -304,131 +421,277 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
       for (int v = 0; v < 5; ++v) Fzm[v] = (R)0;
     }
     idm = ida;
+    put_state(s_qz + tid, NT, QzP);
+#pragma unroll
+    for (int v = 0; v < 5; ++v) s_fz[(5 + v) * NT + tid] = Fzm[v];
+    put(0, cslot, P0, ph[2], id0);
+    put_halo(0, k0);
   }
+  __syncthreads();
+  look_at(0);
+  __syncthreads();
 
   R lam_max = (R)0;
-  const int cslot = (ty + 2) * HX + tx + 2;
 
   for (int k = k0; k < k1; ++k) {
-    const long long pk = (long long)k * nxy;  // k is inside the grid
-    const int buf = SM::NB == 2 ? ((k - k0) & 1) : 0;
-    R* const s_phi = s_phi0 + buf * PL;
-    uint8_t* const s_id = s_id0 + buf * PL;
-    // ---- own column: plane k+2, z face states of cell k+1, z flux of face k+1/2
-    load(plane(k + 2) + own_base, P2, ph[4], id2, own_neg | zneg(k + 2));
-    by_material<MT>(id1, [&](auto T, auto m) {
-      cell_faces<R, GEN, decltype(T)::value>(s_eos[m], P0, P1, P2, id0 == id1 && id2 == id1, QzM1, QzP1, bad, lim,
-                                              alpha);
-    });
-    if (id0 == id1) {
-      num_flux<2, R, GEN>(QzP, QzM1, Fzp, flx);
-    } else {
-#pragma unroll
-      for (int v = 0; v < 5; ++v) Fzp[v] = (R)0;
-    }
-    // ---- plane k into shared memory: own cells and the two-cell halo (no corners)
-#pragma unroll
-    for (int v = 0; v < 5; ++v) s_q[v * PL + cslot] = P0[v];
-    s_phi[cslot] = ph[2];
-    s_id[cslot] = (uint8_t)id0;
-#pragma unroll
-    for (int s = 0; s < HI; ++s) {
-      if (h_hx[s] < 0) break;
-      const int hslot = h_hy[s] * HX + h_hx[s];
-      R Ph[5], phh;
-      int idh;
-      load(pk + halo_base[s], Ph, phh, idh, halo_neg[s]);
-#pragma unroll
-      for (int v = 0; v < 5; ++v) s_q[v * PL + hslot] = Ph[v];
-      s_phi[hslot] = phh;
-      s_id[hslot] = (uint8_t)idh;
-    }
-    __syncthreads();
-
-    // ---- MUSCL face states along x (cells x = -1 .. TX) and y (cells y = -1 .. TY)
-#pragma unroll
-    for (int s = 0; s < SI; ++s) {
-      const int it = st_item(s);
-      if (it < 0) break;
-      const int c0 = it & 1023, so = (it >> 10) ? HX : 1;
-      R Pm[5], P[5], Pp[5];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        Pm[v] = s_q[v * PL + c0 - so];
-        P[v] = s_q[v * PL + c0];
-        Pp[v] = s_q[v * PL + c0 + so];
-      }
-      const int ic = s_id[c0];
-      const bool same = s_id[c0 - so] == ic && s_id[c0 + so] == ic;
-      bool b = false;
-      FaceState<R>* out = s_st + 2 * (tid + s * NT);
-      by_material<MT>(ic, [&](auto T, auto m) {
-        cell_faces<R, GEN, decltype(T)::value>(s_eos[m], Pm, P, Pp, same, out[0], out[1], b, lim, alpha);
-      });
-      bad = bad || b;
-    }
-    __syncthreads();
-
-    // ---- HLLC on every x face (between cells f-1 and f of a row) and y face of the tile
-#pragma unroll
-    for (int s = 0; s < FI; ++s) {
-      int itb;
-      const int it = flux_item(s, itb);
-      if (it < 0) break;
-      const int dir = (it >> 30) & 1;
-      const int lsi = it & 0xffff, idp = itb & 0xffff, outo = (itb >> 16) & 0x7fff;
-      const int il = s_id[idp], ir = s_id[idp + (dir ? HX : 1)];
-      const FaceState<R>& QL = s_st[lsi];
-      const FaceState<R>& QR = s_st[lsi + (dir ? 2 * TX - 1 : 1)];
-      R F[5];
-      if (il != ir) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) F[v] = (R)0;
-      } else if (dir == 0) {
-        num_flux<0, R, GEN>(QL, QR, F, flx);
-      } else {
-        num_flux<1, R, GEN>(QL, QR, F, flx);
-      }
-      R* o = (dir ? s_fy : s_fx) + outo;
-      const int stride = dir ? SFY : SFX;
-#pragma unroll
-      for (int v = 0; v < 5; ++v) o[v * stride] = F[v];
-    }
-    __syncthreads();
-
-    // ---- per cell: residual, level set, Runge-Kutta update, work lists
+    const int pk = k * nxy;  // k is inside the grid
+    const int buf = (k - k0) & 1;
+    const R* const q = s_q + buf * 5 * PL;
+    const R* const phip = s_phi + buf * PL;
+    const uint8_t* const idp = s_id + buf * PL;
+    // faces of the own cell between materials: bits 0, 1 plus x and y, bit 2 any other
+    int iff;
     {
-      const int idxm = s_id[cslot - 1], idxp = s_id[cslot + 1];
-      const int idym = s_id[cslot - HX], idyp = s_id[cslot + HX];
-      const bool is_if = inside && (idxm != id0 || idxp != id0 || idym != id0 || idyp != id0 || idm != id0 ||
-                                    id1 != id0);
-      R res[5];
-      R Fxm[5], Fxp[5], Fym[5], Fyp[5];
+      const int xp = idp[cslot + 1] != id0, yp = idp[cslot + HX] != id0;
+      iff = xp | (yp << 1) | ((idp[cslot - 1] != id0 || idp[cslot - HX] != id0 || idm != id0 || id1 != id0) ? 4 : 0);
+    }
+
+    R* const fz = s_fz + buf * 5 * NT + tid;         // flux through the upper z face
+    const R* const fzm = s_fz + (buf ^ 1) * 5 * NT + tid;  // and the lower one
+
+    // ---- to L2: the row's cells of plane k+4 (loaded two planes from now), and the old state of
+    // plane k+2 where the update reads one besides the stage's; lanes 0 .. 5 and 6 .. 11, a field each
+    if (row_in && tx < (mode == kStage1 || mode == kResidual ? 6 : 12)) {
+      const int f = tx < 6 ? tx : tx - 6, kp = tx < 6 ? k + 4 : k + 2;
+      const double* const a = f == 5 ? (tx < 6 ? phis : G.phi) : (tx < 6 ? Ws : G.W) + f * N;
+      if (kp < nz && kp <= k1 + 1) prefetch_row(a, N, kp * nxy + gy * nx + x0);
+    }
+    // ---- plane k+1 into shared memory: own cells and the two-cell halo (no corners); own
+    // column: plane k+2
+    if (row_on) {
+      put(buf ^ 1, cslot, P1, ph[3], id1);
+      load(plane(k + 2) + own_base, P2, ph[4], id2, own_neg | zneg(k + 2));
+    }
+    if (k + 1 < k1) put_halo(buf ^ 1, k + 1);
+    const R* const qn = s_q + (buf ^ 1) * 5 * PL + cslot;
+
+    // ---- uniform cells and rows; face-state jobs of this warp: bit 0 the plus z state of cell k
+    // where it was left out before, 1 z (cell k+1), 2 x, 3 y, 4 a cell outside the tile
+    bool flat_x = false, flat_y = false, flat_z1 = false, rowflat_z1 = false, need_yp = true;
+    unsigned jobs = 0;
+    if (row_in) {
+      // alike_z: cells k and k+1; a cell is uniform along an axis if it is like both neighbours
+      bool az = is_finite(P1[4]) & (id1 == id2);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        Fxm[v] = s_fx[v * SFX + ty * (TX + 1) + tx];
-        Fxp[v] = s_fx[v * SFX + ty * (TX + 1) + tx + 1];
-        Fym[v] = s_fy[v * SFY + ty * TX + tx];
-        Fyp[v] = s_fy[v * SFY + (ty + 1) * TX + tx];
-        res[v] = ((Fxm[v] - Fxp[v]) * ih + (Fym[v] - Fyp[v]) * ih) + (Fzm[v] - Fzp[v]) * ih;
+      for (int v = 0; v < 5; ++v) az = az & same_bits(P1[v], P2[v]);
+      flat_z1 = alike_z & az;
+      alike_z = az;
+      rowflat_z1 = __all_sync(0xffffffffu, flat_z1);
+      if (!(rowflat_z0 && rowflat_z1)) jobs |= qz_set ? 2u : 3u;
+      qz_set = jobs != 0;
+      // a row's first and last cell count as uniform where the cells outside it were looked at
+      const unsigned m = mx & (mx << 1 | (mx_ends ? 1u : 0u)) & (mx_ends ? 0xffffffffu : 0x7fffffffu);
+      flat_x = (m >> tx) & 1u;
+      if (!mx_ends) jobs |= 4u;
+    }
+    if (row_y) {
+      const unsigned em = s_ey[ty + 1], e0 = s_ey[ty + 2];
+      flat_y = (em & e0) >> tx & 1u;
+      need_yp = (em & e0 & s_ey[ty + 3]) != 0xffffffffu;
+      if (need_yp || s_ey[ty] != 0xffffffffu) jobs |= 8u;
+    }
+    bool out_on = false, out_any = false;  // this lane's cell outside the tile counts, any of the warp's
+    int c_out = cslot, so_out = HX;        // its slot and axis
+    if (ty == kWarpX) {
+      const int row = tx & (TY - 1), hi = tx / TY;
+      out_on = hi < 2 && y0 + row < ny && !s_ex[row];
+      out_any = __any_sync(0xffffffffu, out_on);
+      if (hi < 2) c_out = (row + 2) * HX + (hi ? TX + 2 : 1);
+      so_out = 1;
+    } else if (ty == kWarpY0) {
+      out_on = out_any = (s_ey[0] & s_ey[1] & s_ey[2]) != 0xffffffffu;
+      c_out = HX + tx + 2;
+    } else if (ty == kWarpY1) {
+      out_on = out_any = y0 + TY <= ny && (s_ey[TY] & s_ey[TY + 1] & s_ey[TY + 2]) != 0xffffffffu;
+      c_out = (TY + 2) * HX + tx + 2;
+    }
+    if (out_any) jobs |= 16u;
+    if (mode == kResidual && row_in && (jobs & 14u) == 0) {
+      // no face state will test this cell: its state must be admissible (the stages of a step
+      // test it in the wave-speed sum of the last one)
+      R e, c2;
+      by_material<MT>(id0, [&](auto T, auto m) {
+        const R rho = q[cslot];
+        if (!eos_e_c2<R, GEN, decltype(T)::value>(eos(m), rho, rrcp<R>(rho), q[4 * PL + cslot], e, c2)) bad = true;
+      });
+    }
+
+    // ---- face states
+    FaceState<R> QyP;
+    R Fxp[5] = {(R)0, (R)0, (R)0, (R)0, (R)0};
+#pragma unroll 1
+    for (; jobs; jobs &= jobs - 1) {
+      const int j = __ffs(jobs) - 1;
+      R Pm[5], P[5], Pp[5];
+      int ic;
+      bool same;
+      if (j <= 1) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          Pm[v] = q[v * PL + cslot];
+          P[v] = j ? qn[v * PL] : Pm[v];
+          Pp[v] = j ? P2[v] : Pm[v];
+        }
+        ic = j ? id1 : id0;
+        same = !j || (id0 == id1 && id2 == id1);
+      } else {
+        const int c0 = j == 4 ? c_out : cslot, so = j == 4 ? so_out : (j == 2 ? 1 : HX);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          Pm[v] = q[v * PL + c0 - so];
+          P[v] = q[v * PL + c0];
+          Pp[v] = q[v * PL + c0 + so];
+        }
+        ic = idp[c0];
+        same = idp[c0 - so] == ic && idp[c0 + so] == ic;
+      }
+      FaceState<R> QM, QP;
+      bool b = false;
+      material_faces<GEN, MT, R>(eos, ic, Pm, P, Pp, same, QM, QP, b, lim, alpha);
+      bad = bad || (b && (j < 4 || out_on));
+      if (j <= 1) {
+        if (j == 1) {
+          R F[5];
+          if (id0 == id1) {
+            num_flux<2, R, GEN>(get_state(s_qz + tid, NT), QM, F, flx);
+          } else {
+#pragma unroll
+            for (int v = 0; v < 5; ++v) F[v] = (R)0;
+          }
+#pragma unroll
+          for (int v = 0; v < 5; ++v) fz[v * NT] = F[v];
+        }
+        put_state(s_qz + tid, NT, QP);
+      } else if (j == 2) {
+        // the states of the tile's first and last cell go to the warp that makes the fluxes
+        // through the tile's x faces
+        if (tx == 0) put_state(s_xe + TY + ty, SXE, QM);
+        if (tx == TX - 1) put_state(s_xe + 2 * TY + ty, SXE, QP);
+        FaceState<R> QR;
+        QR.rho = __shfl_down_sync(0xffffffffu, QM.rho, 1);
+        QR.u = __shfl_down_sync(0xffffffffu, QM.u, 1);
+        QR.v = __shfl_down_sync(0xffffffffu, QM.v, 1);
+        QR.w = __shfl_down_sync(0xffffffffu, QM.w, 1);
+        QR.p = __shfl_down_sync(0xffffffffu, QM.p, 1);
+        QR.c = __shfl_down_sync(0xffffffffu, QM.c, 1);
+        QR.E = __shfl_down_sync(0xffffffffu, QM.E, 1);
+        if (!(iff & 1)) num_flux<0, R, GEN>(QP, QR, Fxp, flx);
+      } else if (j == 3) {
+        put_state(s_ym + ty * TX + tx, SYM, QM);
+        QyP = QP;
+      } else if (ty == kWarpX) {
+        if (out_on) {
+          const int row = tx & (TY - 1);
+          if (tx < TY) put_state(s_xe + row, SXE, QP);
+          else put_state(s_xe + 3 * TY + row, SXE, QM);
+        }
+      } else if (ty == kWarpY0) {
+        put_state(s_yp + tx, TX, QP);
+      } else {
+        put_state(s_ym + TY * TX + tx, SYM, QM);
+      }
+    }
+    __syncthreads();
+
+    // ---- y fluxes, the fluxes through the tile's x faces and its lower y face, the level-set residual
+    R Lphi = (R)0;
+    if (row_in) {
+      if (need_yp) {
+        R F[5];
+        if (!(iff & 2)) {
+          num_flux<1, R, GEN>(QyP, get_state(s_ym + (ty + 1) * TX + tx, SYM), F, flx);
+        } else {
+#pragma unroll
+          for (int v = 0; v < 5; ++v) F[v] = (R)0;
+        }
+#pragma unroll
+        for (int v = 0; v < 5; ++v) s_yf[v * SYM + (ty + 1) * TX + tx] = F[v];
       }
       // level-set residual -((u phi_x + v phi_y) + w phi_z), third-order upwind-biased (Sec. 4.4)
-      const R u = P0[1], vv = P0[2], w = P0[3];
-      const R* prow = s_phi + cslot;
-      R Dx, Dy, Dz;
-      if (nonneg(u)) Dx = (((R)2 * prow[1] + (R)3 * prow[0]) - (R)6 * prow[-1] + prow[-2]) * i6h;
-      else Dx = ((-prow[2] + (R)6 * prow[1]) - (R)3 * prow[0] - (R)2 * prow[-1]) * i6h;
-      if (nonneg(vv)) Dy = (((R)2 * prow[HX] + (R)3 * prow[0]) - (R)6 * prow[-HX] + prow[-2 * HX]) * i6h;
-      else Dy = ((-prow[2 * HX] + (R)6 * prow[HX]) - (R)3 * prow[0] - (R)2 * prow[-HX]) * i6h;
-      if (nonneg(w)) Dz = (((R)2 * ph[3] + (R)3 * ph[2]) - (R)6 * ph[1] + ph[0]) * i6h;
-      else Dz = ((-ph[4] + (R)6 * ph[3]) - (R)3 * ph[2] - (R)2 * ph[1]) * i6h;
-      R Lphi = -((u * Dx + vv * Dy) + w * Dz);
+      const R u = q[PL + cslot], vv = q[2 * PL + cslot], w = q[3 * PL + cslot];
+      const R* prow = phip + cslot;
+      // the four values upwind of the cell, mirrored for a negative velocity (FP32: roundings written out)
+      auto deriv = [&](R vel, R m2, R m1, R c, R p1, R p2) {
+        if constexpr (sizeof(R) == 4) {
+          return nonneg(vel) ? __fmul_rn(__fadd_rn(__fmaf_rn(-6.0f, m1, __fmaf_rn(2.0f, p1, __fmul_rn(3.0f, c))), m2), i6h)
+                             : __fmul_rn(__fmaf_rn(-2.0f, m1, __fmaf_rn(-3.0f, c, __fmaf_rn(6.0f, p1, -p2))), i6h);
+        } else {
+          return nonneg(vel) ? ((((R)2 * p1 + (R)3 * c) - (R)6 * m1) + m2) * i6h
+                             : (((-p2 + (R)6 * p1) - (R)3 * c) - (R)2 * m1) * i6h;
+        }
+      };
+      const R Dx = deriv(u, prow[-2], prow[-1], prow[0], prow[1], prow[2]);
+      const R Dy = deriv(vv, prow[-2 * HX], prow[-HX], prow[0], prow[HX], prow[2 * HX]);
+      R Dz = deriv(w, ph[0], ph[1], ph[2], ph[3], ph[4]);
+      if constexpr (sizeof(R) == 4 && !GEN && MT == 0) {
+        // (two stiffened gases: the rounding order of this sum along z that their kernel always had)
+        if (nonneg(w))
+          Dz = __fmul_rn(__fadd_rn(__fmaf_rn(-6.0f, ph[1], __fmaf_rn(3.0f, ph[2], __fmul_rn(2.0f, ph[3]))), ph[0]), i6h);
+      }
+      if constexpr (sizeof(R) == 4) Lphi = -__fmaf_rn(w, Dz, __fmaf_rn(u, Dx, __fmul_rn(vv, Dy)));
+      else Lphi = -((u * Dx + vv * Dy) + w * Dz);
       if constexpr (GEN) {
         // narrow band (Sec. 4.4): the velocity scaled by the cutoff of the cell's level set
         if (G.band_gamma > 0.0) Lphi = band_cutoff<R>((R)G.band_beta, (R)G.band_gamma, ph[2]) * Lphi;
       }
+    }
+    if (ty == kWarpX) {
+      if (out_on) {
+        const int row = tx & (TY - 1), hi = tx / TY;
+        R F[5] = {(R)0, (R)0, (R)0, (R)0, (R)0};
+        const int c0 = (row + 2) * HX + (hi ? TX + 1 : 1);
+        if (idp[c0] == idp[c0 + 1])
+          num_flux<0, R, GEN>(get_state(s_xe + 2 * hi * TY + row, SXE), get_state(s_xe + (2 * hi + 1) * TY + row, SXE),
+                              F, flx);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) s_xf[(2 * v + hi) * TY + row] = F[v];
+      }
+    } else if (ty == kWarpY0) {
+      if (out_any) {
+        R F[5] = {(R)0, (R)0, (R)0, (R)0, (R)0};
+        const int c0 = HX + tx + 2;
+        if (idp[c0] == idp[c0 + HX]) num_flux<1, R, GEN>(get_state(s_yp + tx, TX), get_state(s_ym + tx, SYM), F, flx);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) s_yf[v * SYM + tx] = F[v];
+      }
+    }
+    if (k + 1 < k1) look_at(buf ^ 1);
+    R P0[5];  // (general kernel: the geometric source)
+    if constexpr (GEN) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) P0[v] = q[v * PL + cslot];
+    }
+    __syncthreads();
 
-      const long long c = pk + own_base;
+    // ---- per cell: residual, Runge-Kutta update, work lists
+    if (row_in) {
+      const bool is_if = inside && iff != 0;
+      // fluxes of the axes along which the cell is not uniform (the others' differences vanish)
+      R res[5];
+      R Fxm[5], Fym[5], Fyp[5], Fzm[5], Fzp[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        Fxm[v] = __shfl_up_sync(0xffffffffu, Fxp[v], 1);
+        if (tx == 0) Fxm[v] = s_xf[2 * v * TY + ty];
+        if (tx == TX - 1) Fxp[v] = s_xf[(2 * v + 1) * TY + ty];
+        const R* yf = s_yf + v * SYM + ty * TX + tx;
+        Fxm[v] = flat_x ? (R)0 : Fxm[v];
+        Fxp[v] = flat_x ? (R)0 : Fxp[v];
+        Fym[v] = flat_y ? (R)0 : yf[0];
+        Fyp[v] = flat_y ? (R)0 : yf[TX];
+        Fzm[v] = flat_z0 ? (R)0 : fzm[v * NT];
+        Fzp[v] = flat_z0 ? (R)0 : fz[v * NT];
+        if constexpr (sizeof(R) == 4) {
+          res[v] = __fmaf_rn(Fzm[v] - Fzp[v], ih, __fmaf_rn(Fxm[v] - Fxp[v], ih, __fmul_rn(Fym[v] - Fyp[v], ih)));
+        } else {
+          res[v] = ((Fxm[v] - Fxp[v]) * ih + (Fym[v] - Fyp[v]) * ih) + (Fzm[v] - Fzp[v]) * ih;
+        }
+      }
+      // a row that changes nothing but its level set (plain copies below); for the last stage
+      // its first-stage state must be the old one too
+      const bool still = !GEN && __all_sync(0xffffffffu, flat_x && flat_y && flat_z0);
+
+      const int c = pk + own_base;
       if constexpr (GEN) {
         // spherical / cylindrical forms (Sec. 3.4): S = -(alpha/r) u_r (rho, rho u, rho v,
         // rho w, rho E + p) at the cell centre r = x0 + (i + 1/2) h from the stage state,
@@ -454,11 +717,16 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
           G.resL[c] = to_d<R>(Lphi);
           G.id[c] = (uint8_t)id0;
         } else if (mode == kStage1) {
-          gst(G.phi1 + c, gld(G.phi + c) + dt * to_d<R>(Lphi));
+          gst(G.phi1 + c, fma(dt, to_d<R>(Lphi), gld(G.phi + c)));
           G.id[c] = (uint8_t)id0;
           if (!is_if) {
+            if (still) {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) gst(G.W1 + v * N + c, gld(G.W + v * N + c) + dt * to_d<R>(res[v]));
+              for (int v = 0; v < 5; ++v) gst(G.W1 + v * N + c, gld(G.W + v * N + c));
+            } else {
+#pragma unroll
+              for (int v = 0; v < 5; ++v) gst(G.W1 + v * N + c, fma(dt, to_d<R>(res[v]), gld(G.W + v * N + c)));
+            }
           }
         } else if (GEN && mode == kStage2of3) {
           // TVD RK3, second stage (Sec. 4.3): W2 = (3/4 W + 1/4 W1) + 1/4 dt R(W1)
@@ -487,19 +755,36 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
           G.id[c] = (uint8_t)(id0 | (neg ? 4 : 0));
           if (!is_if) {
             double wn[5];
+            bool kept = still;  // W1 = W: W' = W, and the stage state's wave speeds are the new state's
+            if (still) {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) {
-              wn[v] = rk3      ? (gld(G.W + v * N + c) / 3.0 + 2.0 / 3.0 * gld(G.W2 + v * N + c)) +
-                                2.0 / 3.0 * dt * to_d<R>(res[v])
-                      : f32inc ? fma(0.5, gld(G.W + v * N + c) + gld(G.W1 + v * N + c), to_d<R>(hdt * res[v]))
-                               : 0.5 * (gld(G.W + v * N + c) + (gld(G.W1 + v * N + c) + dt * to_d<R>(res[v])));
-              gst(G.W + v * N + c, wn[v]);
+              for (int v = 0; v < 5; ++v) {
+                wn[v] = gld(G.W + v * N + c);
+                kept = kept && same_bits(wn[v], gld(G.W1 + v * N + c));
+              }
+            }
+            if (!kept) {
+#pragma unroll
+              for (int v = 0; v < 5; ++v) {
+                wn[v] = rk3      ? (gld(G.W + v * N + c) / 3.0 + 2.0 / 3.0 * gld(G.W2 + v * N + c)) +
+                                  2.0 / 3.0 * dt * to_d<R>(res[v])
+                        : f32inc ? fma(0.5, gld(G.W + v * N + c) + gld(G.W1 + v * N + c), to_d<R>(hdt * res[v]))
+                                 : 0.5 * (gld(G.W + v * N + c) + (gld(G.W1 + v * N + c) + dt * to_d<R>(res[v])));
+                gst(G.W + v * N + c, wn[v]);
+              }
             }
             if (!flip) {
               bool ok;
               R lam = (R)0;
               by_material<MT>(id0, [&](auto T, auto m) {
-                lam = wave_sum_v<R, GEN, decltype(T)::value>(G, s_eos[m], s_eosd[m], wn, ok);
+                if (kept) {
+                  R P[5];
+#pragma unroll
+                  for (int v = 0; v < 5; ++v) P[v] = q[v * PL + cslot];
+                  lam = wave_sum_p<R, GEN, decltype(T)::value>(G, eos(m), P, ok);
+                } else {
+                  lam = wave_sum_v<R, GEN, decltype(T)::value>(G, eos(m), eosd(m), wn, ok);
+                }
               });
               bad = bad || !ok;
               lam_max = fmax(lam_max, lam);
@@ -508,7 +793,7 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
         }
       }
       // ---- work lists: warp ballot, one atomic per warp (skipped when the warp has none)
-      const bool fxf = inside && idxp != id0, fyf = inside && idyp != id0, fzf = inside && id1 != id0;
+      const bool fxf = inside && (iff & 1), fyf = inside && (iff & 2), fzf = inside && id1 != id0;
       const int nf = (int)fxf + (int)fyf + (int)fzf;
       if (__any_sync(0xffffffffu, is_if || nf || flip)) {
         {
@@ -583,18 +868,14 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
         }
       }
     }
-    if constexpr (SM::NB == 1) __syncthreads();  // the next plane overwrites s_phi and s_id
 
     // ---- shift the z window
 #pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      P0[v] = P1[v];
-      P1[v] = P2[v];
-      Fzm[v] = Fzp[v];
-    }
+    for (int v = 0; v < 5; ++v) P1[v] = P2[v];
+    flat_z0 = flat_z1;
+    rowflat_z0 = rowflat_z1;
     ph[0] = ph[1]; ph[1] = ph[2]; ph[2] = ph[3]; ph[3] = ph[4];
     idm = id0; id0 = id1; id1 = id2;
-    QzP = QzP1;
   }
   // failures are latched once per tile, with the thread's column at the tile's first plane
   if (bad) latch_error(ctrl, M2C_ENONPHYS, cell_of(G, gx, gy, k0));
@@ -606,20 +887,20 @@ k_stage(const Grid* __restrict__ grids, const long long* __restrict__ tile_begin
 
 // The shared-memory opt-in is a per-device attribute of the kernel: it is set
 // once on every device the calling threads make current.
-template <typename R, int TY, bool GEN, int MT = -1>
+template <typename R, int TY, bool GEN, int MT, bool ONE>
 void stage_smem_setup() {
   static bool done[kMaxDevices] = {};
   const int dev = current_device();
   if (done[dev]) return;
-  cudaFuncSetAttribute(k_stage<R, TY, GEN, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_stage<R, TY, GEN, MT, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)StageSmem<R, TY>::bytes);
   done[dev] = true;
 }
 
-template <typename R, int TY, bool GEN, int MT = -1>
-cudaError_t launch_stage_t(const Grid* grids, const long long* tiles, int ngrid, long long ntiles, int mode,
+template <typename R, int TY, bool GEN, int MT, bool ONE>
+cudaError_t launch_stage_k(const Grid* grids, const long long* tiles, int ngrid, long long ntiles, int mode,
                            const LaunchPlan& lp, cudaStream_t s) {
-  stage_smem_setup<R, TY, GEN, MT>();
+  stage_smem_setup<R, TY, GEN, MT, ONE>();  // (done by the context's set-up, outside captures)
   long long nb = ntiles;
   if (lp.blocks_per_sm > 0) nb = std::min<long long>(ntiles, (long long)lp.blocks_per_sm * sm_count());
   if (nb < 1) nb = 1;
@@ -627,9 +908,27 @@ cudaError_t launch_stage_t(const Grid* grids, const long long* tiles, int ngrid,
     cudaError_t e = cudaMemsetAsync(lp.counter, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
   }
-  k_stage<R, TY, GEN, MT><<<(unsigned)nb, 32 * TY, StageSmem<R, TY>::bytes, s>>>(grids, tiles, ngrid, ntiles, mode,
-                                                                              lp.sched, lp.counter);
+  StageArg<ONE> arg;
+  if constexpr (ONE) arg.grid = *lp.one;
+  k_stage<R, TY, GEN, MT, ONE><<<(unsigned)nb, 32 * TY, StageSmem<R, TY>::bytes, s>>>(arg, grids, tiles, ngrid, ntiles,
+                                                                                    mode, lp.sched, lp.counter);
   return cudaGetLastError();
+}
+
+template <typename R, int TY, bool GEN, int MT = -1>
+cudaError_t launch_stage_t(const Grid* grids, const long long* tiles, int ngrid, long long ntiles, int mode,
+                           const LaunchPlan& lp, cudaStream_t s) {
+  // (FP64: one kernel for grids alone and in batches, whose results are the same bits)
+  if constexpr (sizeof(R) == 4 && !GEN && MT >= 0) {
+    if (lp.one) return launch_stage_k<R, TY, GEN, MT, true>(grids, tiles, ngrid, ntiles, mode, lp, s);
+  }
+  return launch_stage_k<R, TY, GEN, MT, false>(grids, tiles, ngrid, ntiles, mode, lp, s);
+}
+
+template <typename R, int TY, bool GEN, int MT = -1>
+void stage_smem_setup_t() {
+  if constexpr (sizeof(R) == 4 && !GEN && MT >= 0) stage_smem_setup<R, TY, GEN, MT, true>();
+  stage_smem_setup<R, TY, GEN, MT, false>();
 }
 
 // The launch for the material pair of the plan: instantiations with fixed EOS
@@ -653,11 +952,11 @@ cudaError_t launch_stage_pair(const Grid* grids, const long long* tiles, int ngr
 
 template <typename R, int TY>
 void stage_smem_setup_pairs() {
-  stage_smem_setup<R, TY, false, M2C_EOS_SG + 4 * M2C_EOS_SG>();
-  stage_smem_setup<R, TY, false, M2C_EOS_MG + 4 * M2C_EOS_SG>();
-  stage_smem_setup<R, TY, false, M2C_EOS_SG + 4 * M2C_EOS_MG>();
-  stage_smem_setup<R, TY, false, M2C_EOS_MG + 4 * M2C_EOS_MG>();
-  stage_smem_setup<R, TY, false>();
+  stage_smem_setup_t<R, TY, false, M2C_EOS_SG + 4 * M2C_EOS_SG>();
+  stage_smem_setup_t<R, TY, false, M2C_EOS_MG + 4 * M2C_EOS_SG>();
+  stage_smem_setup_t<R, TY, false, M2C_EOS_SG + 4 * M2C_EOS_MG>();
+  stage_smem_setup_t<R, TY, false, M2C_EOS_MG + 4 * M2C_EOS_MG>();
+  stage_smem_setup_t<R, TY, false>();
 }
 
 }  // namespace m2c

@@ -11,8 +11,8 @@ cudaError_t launch_stage_gen(int prec, const Grid* grids, const long long* tiles
 }
 
 void setup_stage_gen() {
-  stage_smem_setup<double, 8, true>();
-  stage_smem_setup<float, 8, true>();
+  stage_smem_setup_t<double, 8, true>();
+  stage_smem_setup_t<float, 8, true>();
 }
 
 }  // namespace m2c
