@@ -192,11 +192,8 @@ __device__ __forceinline__ bool is_finite(float x) { return (bits_of(x) & 0x7f80
 // Wave-speed sum of a state, sum over the axes with more than one cell of
 // |V_d| + c (the CFL reading of the design notes), in precision R (the mixed
 // path takes the time step from FP32 wave speeds of the FP64 state).
-template <typename R, bool EXT = false, int T = -1>
-__device__ __forceinline__ R wave_sum_p(const Grid& g, const EosP<R>& q, const R P[5], bool& ok) {
-  R e, c2;
-  ok = eos_e_c2<R, EXT, T>(q, P[0], rrcp<R>(P[0]), P[4], e, c2);
-  const R cs = ok ? rsqrt_pos<R>(c2) : (R)0;
+template <typename R>
+__device__ __forceinline__ R wave_sum_c(const Grid& g, const R P[5], R cs) {
   R lam = (R)0;
   if (g.active[0]) lam = lam + (fabs(P[1]) + cs);
   if (g.active[1]) lam = lam + (fabs(P[2]) + cs);
@@ -204,8 +201,25 @@ __device__ __forceinline__ R wave_sum_p(const Grid& g, const EosP<R>& q, const R
   return lam;
 }
 template <typename R, bool EXT = false, int T = -1>
+__device__ __forceinline__ R wave_sum_p(const Grid& g, const EosP<R>& q, const R P[5], bool& ok) {
+  R e, c2;
+  ok = eos_e_c2<R, EXT, T>(q, P[0], rrcp<R>(P[0]), P[4], e, c2);
+  return wave_sum_c<R>(g, P, ok ? rsqrt_pos<R>(c2) : (R)0);
+}
+template <typename R, bool EXT = false, int T = -1>
 __device__ __forceinline__ R wave_sum_v(const Grid& g, const EosP<R>& q, const EosDev& qd, const double w[5], bool& ok) {
   R P[5];
+  if constexpr (sizeof(R) == 4) {
+    if (eos_is<T>(q, M2C_EOS_MG)) {
+      const double x[4] = {w[0], w[1], w[2], w[3]};
+      float y[4], c2;
+      d2f_group<4>(x, y);
+      const float inv = rrcp<float>(y[0]);
+      const double rhoe = prim_velocities_f(inv, y[1], y[2], y[3], w[4], P);
+      ok = mg_wave_c2_f<T == M2C_EOS_MG>(q, inv, d2f(rhoe), c2) && pos(y[0]);
+      return wave_sum_c<float>(g, P, ok ? rsqrt_pos<float>(c2) : 0.0f);
+    }
+  }
   const bool okp = cons_to_prim_v<R, EXT, T>(q, qd, w[0], w[1], w[2], w[3], w[4], P);
   const R lam = wave_sum_p<R, EXT, T>(g, q, P, ok);
   ok = ok && okp;

@@ -556,6 +556,29 @@ __device__ __forceinline__ bool mg_e_c2_f(const EosP<float>& q, float inv_rho, f
   return eta < q.eta_max;
 }
 
+// c^2 of a conserved state (1/rho, rho e) in FP32, for the wave speeds of the time step.
+// Its roundings are not those of the load and the faces (e_R' adds its products the other
+// way; FUSED, where the material type is fixed at compile time: e enters its difference
+// with e_R unrounded): one rounding of the largest wave speed moves every cell of the next
+// step by 1e-8, so each kernel keeps the roundings it has.
+template <bool FUSED>
+__device__ __forceinline__ bool mg_wave_c2_f(const EosP<float>& q, float inv_rho, float rhoe, float& c2) {
+  const float eta = __fmaf_rn(-q.rho0, inv_rho, 1.0f);
+  const bool comp = eta > 0.0f;
+  const float k = __fmul_rn(q.K0, eta);
+  const float id = comp ? __fdividef(1.0f, __fmaf_rn(-q.s, eta, 1.0f)) : 1.0f, id2 = __fmul_rn(id, id);
+  float pR = __fmul_rn(k, id2);
+  float dpR = __fmul_rn(__fmul_rn(__fmul_rn(q.K0, __fmaf_rn(comp ? q.s : 0.0f, eta, 1.0f)), id2), id);
+  float eR = __fmaf_rn(__fmul_rn(pR, eta), q.inv_2rho0, q.e0);
+  float deR = comp ? __fmul_rn(__fmaf_rn(k, id2, __fmul_rn(dpR, eta)), q.inv_2rho0)
+                   : __fmul_rn(k, __fmul_rn(2.0f, q.inv_2rho0));
+  if (!comp && !(eta >= q.eta_min)) mg_ref<float>(q, eta, pR, dpR, eR, deR);
+  const float de = FUSED ? __fmaf_rn(rhoe, inv_rho, -eR) : __fsub_rn(__fmul_rn(rhoe, inv_rho), eR);
+  const float p = __fmaf_rn(q.rg, de, pR);
+  c2 = __fmul_rn(__fmaf_rn(p, q.rg, __fmul_rn(__fmaf_rn(-q.rg, deR, dpR), q.rho0)), __fmul_rn(inv_rho, inv_rho));
+  return eta < q.eta_max && c2 > 0.0f && c2 < INFINITY;
+}
+
 // e(rho, p) and c^2(rho, p) together (App. B.3 and App. C.2: c^2 = dp/drho|_e + p/rho^2 dp/de|_rho).
 // False if rho <= 0, c^2 <= 0 or the state is outside the EOS domain.
 template <typename R, bool EXT = false, int T = -1>

@@ -777,7 +777,8 @@ k_stage(const __grid_constant__ StageArg<ONE> arg, const Grid* __restrict__ grid
               bool ok;
               R lam = (R)0;
               by_material<MT>(id0, [&](auto T, auto m) {
-                if (kept) {
+                // (FP32 MG: the wave speeds' p is not the stage state's to the last bit)
+                if (kept && !(sizeof(R) == 4 && eos_is<decltype(T)::value>(eos(m), M2C_EOS_MG))) {
                   R P[5];
 #pragma unroll
                   for (int v = 0; v < 5; ++v) P[v] = q[v * PL + cslot];
