@@ -40,6 +40,37 @@ struct StageSmem {
   static constexpr size_t bytes = (id_off + 2 * PL + 15) / 16 * 16;
 };
 
+// Shared-plane slot of the cell outside the tile whose face states lane tx of warp ty
+// takes (the tile's last three warps: columns -1 and 32, row -1, row TY), and the axis
+// stride so of its neighbours. A lane with no such cell to take (on false: past the two
+// columns of the x warp, or a row beyond the grid, whose slots of a plane are never
+// written) gets the first cell of the tile's row 0, which is always inside the grid, so
+// that what it reads is defined (a material id is used as an index); its result is not.
+template <int TY>
+__host__ __device__ constexpr int outside_slot(int ty, int tx, bool on, int& so) {
+  constexpr int TX = 32, HX = TX + 4;
+  so = ty == TY - 3 ? 1 : HX;
+  if (ty == TY - 3) return on ? ((tx & (TY - 1)) + 2) * HX + (tx / TY ? TX + 2 : 1) : 2 * HX + 2;
+  return (ty == TY - 2 ? 1 : TY + 2) * HX + tx + 2;
+}
+
+// Shared-plane slot of halo load h of a tile (the two-cell ring without corners: four
+// columns of TY rows, padded to whole warps, then four rows of 32); -1: none.
+template <int TY>
+__host__ __device__ constexpr int halo_slot_of(int h) {
+  constexpr int TX = 32, HX = TX + 4, NHX = (4 * TY + 31) / 32 * 32;
+  const int h2 = h - NHX;
+  if (h < 4 * TY) {
+    const int c4 = h / TY;
+    return (h % TY + 2) * HX + (c4 < 2 ? c4 : TX + c4);
+  }
+  if (h2 >= 0 && h2 < 4 * TX) {
+    const int c4 = h2 / TX;
+    return (c4 < 2 ? c4 : TY + c4) * HX + h2 % TX + 2;
+  }
+  return -1;
+}
+
 // Compile-time integer for the material dispatch below (usable in device code).
 template <int V>
 struct IntC {
@@ -207,18 +238,7 @@ k_stage(const __grid_constant__ StageArg<ONE> arg, const Grid* __restrict__ grid
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const unsigned lane = tid & 31, lt = (1u << lane) - 1u;
   // halo cell s of a plane loaded by this thread (two-cell ring without corners): its slot, -1: none
-  auto halo_slot = [&](int s) {
-    const int h = tid + s * NT, h2 = h - NHX;
-    if (h < 4 * TY) {
-      const int c4 = h / TY;
-      return (h % TY + 2) * HX + (c4 < 2 ? c4 : TX + c4);
-    }
-    if (h2 >= 0 && h2 < 4 * TX) {
-      const int c4 = h2 / TX;
-      return (c4 < 2 ? c4 : TY + c4) * HX + h2 % TX + 2;
-    }
-    return -1;
-  };
+  auto halo_slot = [&](int s) { return halo_slot_of<TY>(tid + s * NT); };
 
   // Tiles of all grids of the launch, taken in order by a fixed stride
   // (sched 0) or from an atomic counter (sched 1).
@@ -491,20 +511,17 @@ k_stage(const __grid_constant__ StageArg<ONE> arg, const Grid* __restrict__ grid
       if (need_yp || s_ey[ty] != 0xffffffffu) jobs |= 8u;
     }
     bool out_on = false, out_any = false;  // this lane's cell outside the tile counts, any of the warp's
-    int c_out = cslot, so_out = HX;        // its slot and axis
     if (ty == kWarpX) {
       const int row = tx & (TY - 1), hi = tx / TY;
       out_on = hi < 2 && y0 + row < ny && !s_ex[row];
       out_any = __any_sync(0xffffffffu, out_on);
-      if (hi < 2) c_out = (row + 2) * HX + (hi ? TX + 2 : 1);
-      so_out = 1;
     } else if (ty == kWarpY0) {
       out_on = out_any = (s_ey[0] & s_ey[1] & s_ey[2]) != 0xffffffffu;
-      c_out = HX + tx + 2;
     } else if (ty == kWarpY1) {
       out_on = out_any = y0 + TY <= ny && (s_ey[TY] & s_ey[TY + 1] & s_ey[TY + 2]) != 0xffffffffu;
-      c_out = (TY + 2) * HX + tx + 2;
     }
+    int so_out;  // the axis stride of its neighbours, and its slot
+    const int c_out = outside_slot<TY>(ty, tx, out_on, so_out);
     if (out_any) jobs |= 16u;
     if (mode == kResidual && row_in && (jobs & 14u) == 0) {
       // no face state will test this cell: its state must be admissible (the stages of a step
