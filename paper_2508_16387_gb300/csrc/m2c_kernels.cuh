@@ -120,10 +120,18 @@ __device__ __forceinline__ bool last_stage(int mode) { return mode == kStage2 ||
 // Index of the cell whose state a ghost position i (outside [0, n)) takes:
 // transmissive = the nearest cell (zero gradient), periodic = wrapped, symmetry =
 // the mirror image across the side (its velocity component along the axis is
-// negated by the caller, see mirrored()).
-__device__ __forceinline__ int map_index(int i, int n, int lo_bc, int hi_bc) {
-  if (i < 0) return lo_bc == M2C_BC_PERIODIC ? ((i % n) + n) % n : (lo_bc == M2C_BC_SYMMETRY ? -1 - i : 0);
-  if (i >= n) return hi_bc == M2C_BC_PERIODIC ? i % n : (hi_bc == M2C_BC_SYMMETRY ? 2 * n - 1 - i : n - 1);
+// negated by the caller, see mirrored()). Always a cell of the grid: positions further
+// across a symmetry side than the grid is long (a tile's lanes beyond a small grid, whose
+// results count nowhere) take the last cell the mirror reaches.
+__host__ __device__ __forceinline__ int map_index(int i, int n, int lo_bc, int hi_bc) {
+  if (i < 0) {
+    if (lo_bc == M2C_BC_PERIODIC) return ((i % n) + n) % n;
+    return lo_bc == M2C_BC_SYMMETRY ? (-1 - i < n ? -1 - i : n - 1) : 0;
+  }
+  if (i >= n) {
+    if (hi_bc == M2C_BC_PERIODIC) return i % n;
+    return hi_bc == M2C_BC_SYMMETRY ? (i < 2 * n ? 2 * n - 1 - i : 0) : n - 1;
+  }
   return i;
 }
 

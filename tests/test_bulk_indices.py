@@ -26,3 +26,8 @@ def test_cells_outside_a_tile_read_written_slots(tmp_path):
     """Every slot of the shared plane that the states of cells outside the tile read (the material
     id there is an array index) is one that the plane's loads have written."""
     assert "unwritten slots read 0" in _run(tmp_path, "outside_check")
+
+
+def test_mapped_positions_are_cells_of_the_grid(tmp_path):
+    """A position anywhere in a tile or its halo, however short the axis, maps to a cell of it."""
+    assert "positions outside 0 wrong 0" in _run(tmp_path, "map_check")
