@@ -102,6 +102,29 @@ __device__ __forceinline__ bool cons_to_prim(const EosP<R>& q, const EosDev& qd,
   return cons_to_prim_v<R, EXT>(q, qd, W[c], W[N + c], W[2 * N + c], W[3 * N + c], W[4 * N + c], P);
 }
 
+// FP64 primitive state of a cell of material m in the kernels beside the bulk kernel (interface
+// faces and cells, phase update, conversions): the KEPT arithmetic for a mixed grid.
+__device__ __forceinline__ bool cell_prims(const Grid& g, int m, const double* __restrict__ W, long long c, double P[5]) {
+  const EosDev& q = g.eos[m];
+  const long long N = g.N;
+  if (g.prec != M2C_MIXED) return cons_to_prim<double, true>(q, q, W, N, c, P);
+  const double rho = W[c], m1 = W[N + c], m2 = W[2 * N + c], m3 = W[3 * N + c], E = W[4 * N + c];
+  const double inv = rcp_kept(rho);
+  const double u = m1 * inv, v = m2 * inv, w = m3 * inv;
+  const double ke = 0.5 * ((m1 * u + m2 * v) + m3 * w);
+  const double e = (E - ke) * inv;
+  double p = 0.0;
+  const bool ok = eos_p_kept(q, rho, inv, e, p);
+  P[0] = rho; P[1] = u; P[2] = v; P[3] = w; P[4] = p;
+  return ok && gt0(rho);
+}
+// e of a state (rho, p) in the same kernels; false if it is not admissible.
+__device__ __forceinline__ bool cell_energy(const Grid& g, int m, double rho, double p, double& e) {
+  double c2;
+  return g.prec == M2C_MIXED ? eos_e_c2_kept(g.eos[m], rho, 1.0 / rho, p, e, c2)
+                             : eos_e_c2<double, true>(g.eos[m], rho, 1.0 / rho, p, e, c2);
+}
+
 // e and c^2 of an FP32 face state (mixed path) for a material type fixed at compile
 // time: no branches, every rounding written out, so that the face states do not
 // depend on how the compiler contracts them in each kernel. False if not admissible.

@@ -335,13 +335,17 @@ __device__ __forceinline__ bool nr_range_pos(double b) { return hi_of(b) - 0x382
 static __device__ __noinline__ double rcp_ieee(double b) { return 1.0 / b; }
 static __device__ __noinline__ double div_ieee(double a, double b) { return a / b; }
 static __device__ __noinline__ double sqrt_ieee(double x) { return sqrt(x); }
-__device__ __forceinline__ double rcp_nr_in_range(double b) {
+// binary32 seed of 1/b, b in the Newton range
+__device__ __forceinline__ double rcp_seed(double b) {
   const unsigned hi = hi_of(b), ah = hi & 0x7fffffffu;
   const float f = float_of((((ah - 0x38000000u) << 3) | (lo_of(b) >> 29)) | (hi & 0x80000000u));
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
   const unsigned rb = bits_of(r), ra = rb & 0x7fffffffu;
-  const double x = double_of_words(((ra >> 3) + (896u << 20)) | (rb & 0x80000000u), ra << 29);
+  return double_of_words(((ra >> 3) + (896u << 20)) | (rb & 0x80000000u), ra << 29);
+}
+__device__ __forceinline__ double rcp_nr_in_range(double b) {
+  const double x = rcp_seed(b);
   const double e = fma(-b, x, 1.0);
   return fma(x, fma(e, e, e), x);
 }
@@ -416,14 +420,54 @@ __device__ __forceinline__ bool nonneg(R x) {
   else return x >= (R)0;
 }
 
+// FP64 reciprocal, reciprocal root and quotient of the mixed path's interface (the KEPT
+// functions here and in the Riemann solver): the seeds of rcp_nr and rsqrt_nr with two
+// Newton-Raphson steps x <- x + x (1 - b x) and y <- y + y (1 - x y^2)/2. A mixed grid
+// rounds its interface states to binary32 before they become fluxes, and Mie-Grueneisen
+// water turns one such rounding into 130 Pa: states that differ in the last bits of 64
+// then move cells by up to 1e-7. Its interface therefore keeps the arithmetic that its
+// results have always had, operation by operation; FP64 grids and Riemann batches, whose
+// results follow the last bits only, take the shorter forms. Kept on their own operands
+// (fused or not) by comparing whole runs bit for bit.
+__device__ __forceinline__ double rcp_kept_in_range(double b) {
+  const double x0 = rcp_seed(b);
+  const double x = fma(x0, fma(-b, x0, 1.0), x0);
+  return fma(x, fma(-b, x, 1.0), x);
+}
+__device__ __forceinline__ double rcp_kept(double b) {
+  if (nr_range(b)) return rcp_kept_in_range(b);
+  return rcp_ieee(b);
+}
+// x / 2 of a normal x whose half is normal, and x < b for b > 0: on the words
+__device__ __forceinline__ double half_of(double x) { return double_of_words(hi_of(x) - 0x00100000u, lo_of(x)); }
+__device__ __forceinline__ bool lt_pos(double x, double b) { return (long long)bits_of(x) < (long long)bits_of(b); }
+__device__ __forceinline__ double rsqrt_kept(double x) {
+  if (!nr_range_pos(x)) return rcp_ieee(sqrt_ieee(x));
+  double y = rsqrt_seed(x);
+  y = fma(half_of(y), fma(-x * y, y, 1.0), y);
+  y = fma(half_of(y), fma(-x * y, y, 1.0), y);
+  return y;
+}
+__device__ __forceinline__ double div_kept(double a, double b) {
+  if (nr_range(b)) {
+    const double x = rcp_kept_in_range(b), q = a * x;
+    const unsigned ha = hi_of(a), ea = (ha >> 20) & 0x7ffu;
+    if (ea - 126u < 1795u) return fma(fma(-b, q, a), x, q);
+    if (((ha & 0x7fffffffu) | lo_of(a)) == 0u) return q;
+  }
+  return div_ieee(a, b);
+}
+
 // Reference curves p_R, p_R', e_R, e_R' at strain eta (App. B.3); "p_H" in the
 // compression e_R is read as p_R.
-template <typename R>
+template <typename R, bool KEPT = false>
 __device__ __forceinline__ void mg_ref(const EosP<R>& q, R eta, R& pR, R& dpR, R& eR, R& deR) {
   const R K0 = q.K0, rho0 = q.rho0, e0 = q.e0, h2 = q.inv_2rho0;
   if (pos(eta)) {
     R d = (R)1 - q.s * eta;
-    R id = rrcp<R>(d);
+    R id;
+    if constexpr (KEPT) id = rcp_kept(d);
+    else id = rrcp<R>(d);
     R id2 = id * id;
     pR = K0 * eta * id2;
     dpR = K0 * ((R)1 + q.s * eta) * id2 * id;
@@ -613,6 +657,46 @@ __device__ __forceinline__ bool eos_e_c2(const EosP<R>& q, R rho, R inv_rho, R p
   }
   if constexpr (sizeof(R) == 8) return gt0(c2) && hi_of(c2) < 0x7ff00000u;
   else return c2 > (R)0 && c2 < (R)INFINITY;
+}
+
+// The KEPT forms of p(rho, e) and of e, c^2 (rho, p) in FP64 (see rcp_kept): those of a
+// mixed grid's interface, phase update and conversions. NASG and JWL have one form.
+__device__ __forceinline__ bool eos_p_kept(const EosP<double>& q, double rho, double inv_rho, double e, double& p) {
+  if (q.type == M2C_EOS_SG) {
+    p = q.gm1 * rho * e - q.gpc;
+    return true;
+  }
+  if (q.type != M2C_EOS_MG) return eos_p<double, true>(q, rho, inv_rho, e, p);
+  double eta = 1.0 - q.rho0 * inv_rho;
+  if (!(eta < q.eta_max)) return false;
+  double pR, dpR, eR, deR;
+  mg_ref<double, true>(q, eta, pR, dpR, eR, deR);
+  p = pR + q.rg * (e - eR);
+  return true;
+}
+__device__ __forceinline__ bool mg_e_c2_kept(const EosP<double>& q, double rho, double inv_rho, double p, double& e,
+                                             double& c2) {
+  if (!gt0(rho)) return false;
+  double eta = 1.0 - q.rho0 * inv_rho;
+  if (!lt_pos(eta, q.eta_max)) return false;
+  double pR, dpR, eR, deR;
+  mg_ref<double, true>(q, eta, pR, dpR, eR, deR);
+  e = eR + (p - pR) * q.inv_rg;
+  double ir2 = inv_rho * inv_rho;
+  c2 = ((dpR - q.rg * deR) * q.rho0 + p * q.rg) * ir2;
+  return gt0(c2) && hi_of(c2) < 0x7ff00000u;
+}
+__device__ __forceinline__ bool eos_e_c2_kept(const EosP<double>& q, double rho, double inv_rho, double p, double& e,
+                                              double& c2) {
+  if (q.type == M2C_EOS_SG) {
+    if (!gt0(rho)) return false;
+    double pb = p + q.pc;
+    e = (p + q.gpc) * q.inv_gm1 * inv_rho;
+    c2 = q.g * pb * inv_rho;
+    return gt0(c2) && hi_of(c2) < 0x7ff00000u;
+  }
+  if (q.type == M2C_EOS_MG) return mg_e_c2_kept(q, rho, inv_rho, p, e, c2);
+  return eos_e_c2<double, true>(q, rho, inv_rho, p, e, c2);
 }
 
 // ---------------------------------------------------------------------------

@@ -16,6 +16,14 @@ namespace m2c {
 // rarefaction by RK4 on equal pressure substeps whose number is fixed once
 // per problem (fix_substeps) from a bound of the wave's pressure span.
 // ---------------------------------------------------------------------------
+// KEPT (template parameter below): the arithmetic of a mixed grid's interface (rcp_kept in
+// m2c_physics.cuh says why it is kept), in the same control flow: IEEE roots and quotients,
+// two-step reciprocals, the general e and c^2 along the isentrope, the PVRS start. Without
+// it, the shorter forms of FP64 grids and Riemann batches. What it costs: a FIVER launch of
+// a late shock-bubble takes 2300 us at 192^3 and 1270 at 131x67x45, against 980 and 312 with
+// the shorter forms (3188 and 1733 with the kept arithmetic before the control flow was made
+// reconvergent): 35 FP64 instructions instead of 16 in the isentrope's right-hand side, and
+// faces without a previous star pressure take 13 Newton iterations from the PVRS estimate.
 constexpr double kNewtonTol = 1e-12;
 constexpr int kNewtonCap = 50;
 constexpr int kBisectCap = 200;
@@ -40,16 +48,28 @@ struct Side {
   double dnode, idnode, dspan, rbase, fbase, rprev, fprev;  // dspan = nrk dnode, the span bound the nodes cover
 };
 
+template <bool KEPT>
 __device__ inline bool make_side(const EosDev& q, double rho, double u, double p, Side& K) {
-  double e = 0.0, c2 = 0.0;
-  const double iv = rcp_nr(rho);
-  if (!eos_e_c2<double, true>(q, rho, iv, p, e, c2)) return false;
+  double e = 0.0, c2 = 0.0, iv;
+  if constexpr (KEPT) {
+    if (!eos_e_c2_kept(q, rho, 1.0 / rho, p, e, c2)) return false;
+    K.c = sqrt(c2);
+    iv = div_kept(1.0, rho);
+  } else {
+    iv = rcp_nr(rho);
+    if (!eos_e_c2<double, true>(q, rho, iv, p, e, c2)) return false;
+    K.c = sqrt_nr(c2);
+  }
   K.rho = rho;
   K.u = u;
   K.p = p;
-  K.c = sqrt_nr(c2);
   K.e = e;
-  if (q.type == M2C_EOS_SG) {
+  if (q.type == M2C_EOS_SG && KEPT) {
+    K.pb = p + q.pc;
+    K.z = rho * K.c;
+    K.cf = 2.0 * K.c / (q.g - 1.0);
+    K.A = 2.0 / ((q.g + 1.0) * rho);
+  } else if (q.type == M2C_EOS_SG) {
     K.pb = p + q.pc;
     K.ipb = rcp_nr(K.pb);
     K.z = rho * K.c;
@@ -58,7 +78,7 @@ __device__ inline bool make_side(const EosDev& q, double rho, double u, double p
     K.B = q.gm * K.pb;
   } else {
     K.iv = iv;
-    K.ic2 = rcp_nr(c2);
+    if constexpr (!KEPT) K.ic2 = rcp_nr(c2);
     K.hp = NAN;
     K.nrk = 0;
     K.mbase = 0;
@@ -137,9 +157,22 @@ struct Wave {
 // branch and loop: with returns inside the loops a warp executed 12-15 Newton
 // iterations and 90-140 isentrope substeps for an average of 3 and 30 a face
 // (late shock-bubble), the lanes taking turns.
+template <bool KEPT>
 __device__ inline int wave_sg(const EosDev& q, const Side& K, double p, Wave& w) {
   const double pb = p + q.pc, dp = p - K.p;
-  if (p > K.p) {
+  if constexpr (KEPT) {
+    if (p > K.p) {
+      const double B = q.gm * K.pb;
+      const double sq = sqrt(K.A / (pb + B));
+      w.f = (p - K.p) * sq;
+      w.df = sq * (1.0 - 0.5 * (p - K.p) / (pb + B));
+    } else {
+      const double r = pb / K.pb;
+      const double pw = pow(r, q.ex);
+      w.f = K.cf * (pw - 1.0);
+      w.df = pw / (r * K.rho * K.c);
+    }
+  } else if (p > K.p) {
     // f = dp sqrt(A/(pb + B)), f' = sqrt(A/(pb + B)) (1 - dp/(2 (pb + B)))
     const double iD = rcp_nr(pb + K.B), sq = sqrt_nr(K.A * iD);
     w.f = dp * sq;
@@ -160,7 +193,42 @@ __device__ inline int wave_sg(const EosDev& q, const Side& K, double p, Wave& w)
 // in a closed bracket, stopped at the first step below the tolerance) and
 // d rho/dp along it. The start is the root of the problem's previous evaluation
 // moved along its slope, else the acoustic density.
+template <bool KEPT>
 __device__ inline int mg_hugoniot(const EosDev& q, Side& K, double p, double& rho_out, double& drdp) {
+  if constexpr (KEPT) {
+    double lo = K.rho, hi = q.rmax;
+    bool more = hi > lo;
+    int st = more ? M2C_OK : M2C_ENONPHYS;
+    double rho = K.rho + div_kept(p - K.p, K.c * K.c);
+    if (!(rho > lo && rho < hi)) rho = 0.5 * (lo + hi);
+    for (int it = 0; more; ++it) {
+      const double ir = div_kept(1.0, rho), eta = 1.0 - div_kept(q.rho0, rho);
+      double pR = 0.0, dpR = 0.0, eR = 0.0, deR = 0.0;
+      mg_ref<double, true>(q, eta, pR, dpR, eR, deR);
+      double e = eR + (p - pR) * q.inv_rg;
+      double dedr = div_kept((deR - dpR * q.inv_rg) * q.rho0, rho * rho);
+      double H = e - K.e - 0.5 * (p + K.p) * (K.iv - ir);
+      double dH = dedr - div_kept(0.5 * (p + K.p), rho * rho);
+      if (H > 0.0) lo = rho; else hi = rho;
+      double rn = rho - div_kept(H, dH);
+      if (!(rn >= lo && rn <= hi)) rn = 0.5 * (lo + hi);
+      const bool conv = fabs(rn - rho) <= kHugTol * rn;
+      rho = rn;
+      if (!(eta < q.eta_max)) st = M2C_ENONPHYS;
+      else if (!conv && it + 1 == kHugCap) st = M2C_ENOCONV;
+      more = st == M2C_OK && !conv;
+    }
+    const double eta = 1.0 - div_kept(q.rho0, rho);
+    if (!st && !(eta < q.eta_max)) st = M2C_ENONPHYS;
+    double pR = 0.0, dpR = 0.0, eR = 0.0, deR = 0.0;
+    mg_ref<double, true>(q, eta, pR, dpR, eR, deR);
+    const double dedr = div_kept((deR - dpR * q.inv_rg) * q.rho0, rho * rho);
+    double Hp = q.inv_rg - 0.5 * (K.iv - div_kept(1.0, rho));
+    double Hr = dedr - div_kept(0.5 * (p + K.p), rho * rho);
+    rho_out = rho;
+    drdp = -div_kept(Hp, Hr);
+    return st;
+  }
   double lo = K.rho, hi = q.rmax;
   bool more = hi > lo;
   int st = more ? M2C_OK : M2C_ENONPHYS;
@@ -218,6 +286,28 @@ __device__ inline void mg_rhs(const EosDev& q, double g, double rho, double& kr,
   kr = ry * ry;
 }
 
+// The same in the kept arithmetic: d rho/dp = 1/c^2 and df/dp = 1/(rho c) from one
+// reciprocal square root of the general c^2 and the reciprocal of rho.
+__device__ inline void mg_rhs_kept(const EosDev& q, double p, double rho, double& drho, double& dfv, bool& ok) {
+  double e, c2 = 1.0;
+  const double ir = rcp_kept(rho);
+  ok = mg_e_c2_kept(q, rho, ir, p, e, c2) && ok;
+  const double y = rsqrt_kept(c2);
+  drho = y * y;
+  dfv = y * ir;
+}
+// (h6: hs / 6, rounded)
+__device__ inline void mg_rk4_substep_kept(const EosDev& q, double pi, double hs, double h6, double& rho, double& fv,
+                                           bool& ok) {
+  double k1r, k1f, k2r, k2f, k3r, k3f, k4r, k4f;
+  mg_rhs_kept(q, pi, rho, k1r, k1f, ok);
+  mg_rhs_kept(q, pi + 0.5 * hs, rho + 0.5 * hs * k1r, k2r, k2f, ok);
+  mg_rhs_kept(q, pi + 0.5 * hs, rho + 0.5 * hs * k2r, k3r, k3f, ok);
+  mg_rhs_kept(q, pi + hs, rho + hs * k3r, k4r, k4f, ok);
+  rho = rho + h6 * (k1r + 2.0 * k2r + 2.0 * k3r + k4r);
+  fv = fv + h6 * (k1f + 2.0 * k2f + 2.0 * k3f + k4f);
+}
+
 // One classical RK4 substep of the MG isentrope (rho, f) from pressure pi by hs.
 __device__ inline void mg_rk4_substep(const EosDev& q, double pi, double hs, double& rho, double& fv, bool& ok) {
   const double g0 = q.gk * pi, gh = q.gk * hs, gm = fma(0.5, gh, g0);
@@ -241,16 +331,26 @@ __device__ inline void mg_rk4_substep(const EosDev& q, double pi, double hs, dou
 // alone, equal substeps over p_K - p. All are one loop, so that the lanes of a
 // warp take their substeps together. The node arithmetic is written without
 // contracted multiply-adds, so that it takes the same nodes as the oracle.
+template <bool KEPT>
 __device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
   int st = M2C_OK;
   if (p == K.p) {
     w.f = 0.0;
-    w.df = K.iv * rcp_nr(K.c);
+    w.df = KEPT ? 1.0 / (K.rho * K.c) : K.iv * rcp_nr(K.c);
     w.a = K.rho;
-    w.b = K.ic2;
+    w.b = KEPT ? 1.0 / (K.c * K.c) : K.ic2;
+  } else if (p > K.p && KEPT) {
+    double rho, drdp;
+    st = mg_hugoniot<KEPT>(q, K, p, rho, drdp);
+    double dv = K.iv - div_kept(1.0, rho);
+    double fv = sqrt((p - K.p) * dv);
+    w.f = fv;
+    w.df = div_kept(dv + div_kept((p - K.p) * drdp, rho * rho), 2.0 * fv);
+    w.a = rho;
+    w.b = drdp;
   } else if (p > K.p) {
     double rho, drdp;
-    st = mg_hugoniot(q, K, p, rho, drdp);
+    st = mg_hugoniot<KEPT>(q, K, p, rho, drdp);
     const double ir = rcp_nr(rho), dv = K.iv - ir, dp = p - K.p;
     const double fv = sqrt_nr(dp * dv);
     w.f = fv;
@@ -259,12 +359,17 @@ __device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
     w.b = drdp;
   } else {
     const double dp = __dsub_rn(K.p, p);
-    const bool within = K.nrk > 1 && K.dnode > 0.0 && dp < K.dspan + K.dnode;
+    // (kept: beyond the bound itself, equal substeps)
+    const bool within = K.nrk > 1 && K.dnode > 0.0 && dp < (KEPT ? K.dspan : K.dspan + K.dnode);
     double rho = K.rho, fv = 0.0, gap = 0.0, last = dp;
     int i = 0, m = 0;
     if (within) {
-      const double m0 = dp * K.idnode;
-      m = (int)floor(fma(fma(-K.dnode, m0, dp), K.idnode, m0));  // the IEEE quotient dp/dnode
+      if constexpr (KEPT) {
+        m = (int)floor(div_kept(dp, K.dnode));
+      } else {
+        const double m0 = dp * K.idnode;
+        m = (int)floor(fma(fma(-K.dnode, m0, dp), K.idnode, m0));  // the IEEE quotient dp/dnode
+      }
       m = min(m, dp < K.dspan ? K.nrk - 1 : K.nrk);
       if (K.mbase <= m) {
         i = K.mbase;
@@ -282,17 +387,23 @@ __device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
       const int ns = K.nrk > 0 ? K.nrk : mg_substeps(q, dp);
       if (ns > 1) {
         m = ns;
-        gap = div_nr(dp, (double)ns);
+        gap = KEPT ? (K.p - p) / ns : div_nr(dp, (double)ns);
         last = 0.0;
       }
     }
     bool ok = true;
     if (i < m) {
       double rp = rho, fp = fv;
+      const double h6 = KEPT ? -gap / 6.0 : 0.0;
       for (; i < m; ++i) {
         rp = rho;
         fp = fv;
-        mg_rk4_substep(q, __dsub_rn(K.p, __dmul_rn((double)i, gap)), -gap, rho, fv, ok);
+        if constexpr (KEPT) {
+          const double pi = within ? __dsub_rn(K.p, __dmul_rn((double)i, gap)) : fma((double)i, -gap, K.p);
+          mg_rk4_substep_kept(q, pi, -gap, h6, rho, fv, ok);
+        } else {
+          mg_rk4_substep(q, __dsub_rn(K.p, __dmul_rn((double)i, gap)), -gap, rho, fv, ok);
+        }
       }
       if (within) {
         K.mbase = m;
@@ -304,13 +415,23 @@ __device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
     }
     const double pm = __dmul_rn((double)m, gap);
     if (within) last = __dsub_rn(dp, pm);
-    if (last > 0.0) mg_rk4_substep(q, __dsub_rn(K.p, pm), -last, rho, fv, ok);
-    double k, y;
-    mg_rhs(q, q.gk * p, rho, k, y, ok);
-    w.f = fv;
-    w.df = y * q.kap;
-    w.a = rho;
-    w.b = k * q.kap2;
+    if constexpr (KEPT) {
+      if (last > 0.0) mg_rk4_substep_kept(q, __dsub_rn(K.p, pm), -last, -last / 6.0, rho, fv, ok);
+      double e, c2 = 1.0;
+      ok = mg_e_c2_kept(q, rho, 1.0 / rho, p, e, c2) && ok;
+      w.f = fv;
+      w.df = 1.0 / (rho * sqrt(c2));
+      w.a = rho;
+      w.b = 1.0 / c2;
+    } else {
+      if (last > 0.0) mg_rk4_substep(q, __dsub_rn(K.p, pm), -last, rho, fv, ok);
+      double k, y;
+      mg_rhs(q, q.gk * p, rho, k, y, ok);
+      w.f = fv;
+      w.df = y * q.kap;
+      w.a = rho;
+      w.b = k * q.kap2;
+    }
     if (!ok) st = M2C_ENONPHYS;
   }
   return st;
@@ -452,18 +573,29 @@ static __device__ __noinline__ int wave_jwl(const EosDev& q, const Side& K, doub
 }
 
 // A side's wave curve at p; out of line, one copy for both sides.
+template <bool KEPT>
 static __device__ __noinline__ int wave(const EosDev& q, Side& K, double p, Wave& w) {
-  if (q.type == M2C_EOS_SG) return wave_sg(q, K, p, w);
-  if (q.type == M2C_EOS_MG) return wave_mg(q, K, p, w);
+  if (q.type == M2C_EOS_SG) return wave_sg<KEPT>(q, K, p, w);
+  if (q.type == M2C_EOS_MG) return wave_mg<KEPT>(q, K, p, w);
   if (q.type == M2C_EOS_NASG) return wave_nasg(q, K, p, w);
   return wave_jwl(q, K, p, w);
 }
 
 // Density behind the wave w evaluated at p, and its slope d rho*/dp.
+template <bool KEPT>
 __device__ inline void star_density(const EosDev& q, const Side& K, double p, const Wave& w, double& rs, double& drs) {
   if (q.type != M2C_EOS_SG) {
     rs = w.a;
     drs = w.b;
+  } else if (KEPT) {
+    const double gm = q.gm, pb = p + q.pc, r = pb / K.pb;
+    if (p > K.p) {
+      rs = K.rho * (r + gm) / (gm * r + 1.0);
+      drs = K.rho * (1.0 - gm * gm) / ((gm * r + 1.0) * (gm * r + 1.0) * K.pb);
+    } else {
+      rs = K.rho * pow(r, q.inv_g);
+      drs = rs / (q.g * pb);
+    }
   } else if (p > K.p) {
     const double r = (p + q.pc) * K.ipb, id = rcp_nr(fma(q.gm, r, 1.0));
     rs = K.rho * (r + q.gm) * id;
@@ -477,10 +609,11 @@ __device__ inline void star_density(const EosDev& q, const Side& K, double p, co
 }
 
 // F(p) = f_L + f_R + (u_R - u_L) of the bisection and the vacuum test.
+template <bool KEPT>
 static __device__ __noinline__ int riemann_F(const EosDev& qL, Side& L, const EosDev& qR, Side& Rs, double p, double& F) {
   Wave wL, wR;
-  int st = wave(qL, L, p, wL);
-  if (!st) st = wave(qR, Rs, p, wR);
+  int st = wave<KEPT>(qL, L, p, wL);
+  if (!st) st = wave<KEPT>(qR, Rs, p, wR);
   if (!st) F = wL.f + wR.f + (Rs.u - L.u);
   return st;
 }
@@ -492,6 +625,7 @@ struct RiemannOut {
 // A problem whose Newton iteration ran out of steps: the vacuum test, then
 // bisection for p* (iters counts its steps too). Then, and for a converged
 // problem with a slope that is not finite, the star state from an evaluation at p.
+template <bool KEPT>
 static __device__ __noinline__ int riemann_finish(const EosDev& qL, Side& L, const EosDev& qR, Side& Rs, double plow,
                                                   bool vacuum_test, bool conv, double p, RiemannOut& out, int& iters) {
   int st;
@@ -499,7 +633,7 @@ static __device__ __noinline__ int riemann_finish(const EosDev& qL, Side& L, con
   if (!conv) {
     ++iters;
     if (vacuum_test) {
-      st = riemann_F(qL, L, qR, Rs, plow, F);
+      st = riemann_F<KEPT>(qL, L, qR, Rs, plow, F);
       if (st) return st;
       if (F >= 0.0) return M2C_EVACUUM;
     }
@@ -507,14 +641,14 @@ static __device__ __noinline__ int riemann_finish(const EosDev& qL, Side& L, con
     if (!isfinite(a)) {
       a = fmin(L.p, Rs.p);
       for (int k = 0; k < kBisectCap; ++k) {
-        st = riemann_F(qL, L, qR, Rs, a, F);
+        st = riemann_F<KEPT>(qL, L, qR, Rs, a, F);
         if (st) return st;
         if (F < 0.0) break;
         a = a - 2.0 * fabs(a) - 1.0;
       }
     }
     for (int k = 0; k < kBisectCap; ++k) {
-      st = riemann_F(qL, L, qR, Rs, b, F);
+      st = riemann_F<KEPT>(qL, L, qR, Rs, b, F);
       if (st) return st;
       if (F > 0.0) break;
       b = 2.0 * b + fabs(b) + 1.0;
@@ -522,7 +656,7 @@ static __device__ __noinline__ int riemann_finish(const EosDev& qL, Side& L, con
     bool ok = false;
     for (int k = 0; k < kBisectCap; ++k) {
       double m = 0.5 * (a + b);
-      st = riemann_F(qL, L, qR, Rs, m, F);
+      st = riemann_F<KEPT>(qL, L, qR, Rs, m, F);
       if (st) return st;
       if (F < 0.0) a = m; else b = m;
       ++iters;
@@ -533,13 +667,13 @@ static __device__ __noinline__ int riemann_finish(const EosDev& qL, Side& L, con
   }
   Wave wL, wR;
   double d;
-  st = wave(qL, L, p, wL);
-  if (!st) st = wave(qR, Rs, p, wR);
+  st = wave<KEPT>(qL, L, p, wL);
+  if (!st) st = wave<KEPT>(qR, Rs, p, wR);
   if (st) return st;
   out.p = p;
   out.u = 0.5 * (L.u + Rs.u) + 0.5 * (wR.f - wL.f);
-  star_density(qL, L, p, wL, out.rhoL, d);
-  star_density(qR, Rs, p, wR, out.rhoR, d);
+  star_density<KEPT>(qL, L, p, wL, out.rhoL, d);
+  star_density<KEPT>(qR, Rs, p, wR, out.rhoR, d);
   return M2C_OK;
 }
 
@@ -574,7 +708,8 @@ __device__ inline void guess_wave(const GuessSide& K, float p, float& f, float& 
 // acoustic pressure p_ac. NaN where that fails. The PVRS estimate is far off p*
 // when the sides' impedances differ (water against air) and takes 13
 // iterations, three of them over the whole isentrope; one such face held up its
-// launch (1.51 against 0.59 ms in the late shock-bubble, 131x67x45).
+// launch (1.51 against 0.59 ms in the late shock-bubble, 131x67x45, before mixed grids
+// went back to the kept arithmetic; FP64 grids take it).
 static __device__ __noinline__ double start_guess(const EosDev& qL, const Side& L, const EosDev& qR, const Side& Rs,
                                                   double plow, double pac) {
   if ((qL.type != M2C_EOS_SG && qL.type != M2C_EOS_MG) || (qR.type != M2C_EOS_SG && qR.type != M2C_EOS_MG)) return NAN;
@@ -598,12 +733,13 @@ static __device__ __noinline__ double start_guess(const EosDev& qL, const Side& 
 // PVRS estimate, or, with `guess`, start_guess() where the PVRS estimate and the
 // acoustic pressure differ by more than 5 %. The root and the stopping rule do
 // not depend on the start.
+template <bool KEPT>
 static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, double ul, double pl, const EosDev& qR, double rr,
                                     double ur, double pr, RiemannOut& out, int& iters,
                                     double p_start = NAN, bool guess = false) {
   Side L, Rs;
   iters = 0;
-  if (!make_side(qL, rl, ul, pl, L) || !make_side(qR, rr, ur, pr, Rs)) return M2C_ENONPHYS;
+  if (!make_side<KEPT>(qL, rl, ul, pl, L) || !make_side<KEPT>(qR, rr, ur, pr, Rs)) return M2C_ENONPHYS;
   const double plow = fmax(eos_plow(qL), eos_plow(qR));
   const double pac = fix_substeps(qL, L, qR, Rs, plow);
   int st = M2C_OK;
@@ -619,7 +755,7 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
   const bool warm = p_start > plow && p_start < INFINITY;
   if (warm) {
     p = p_start;
-  } else if (guess && !(fabs(p - pac) <= 0.05 * fabs(pac))) {
+  } else if (!KEPT && guess && !(fabs(p - pac) <= 0.05 * fabs(pac))) {
     const double pg = start_guess(qL, L, qR, Rs, plow, pac);
     if (pg > plow) p = pg;
   }
@@ -637,10 +773,11 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
   int it = 0;
   while (more) {
     ++it;
-    st = wave(qL, L, p, wL);
-    const int sr = wave(qR, Rs, p, wR);
+    st = wave<KEPT>(qL, L, p, wL);
+    const int sr = wave<KEPT>(qR, Rs, p, wR);
     if (!st) st = sr;
-    double pn = p - div_nr(wL.f + wR.f + (Rs.u - L.u), wL.df + wR.df);
+    const double F = wL.f + wR.f + (Rs.u - L.u), dF = wL.df + wR.df;
+    double pn = p - (KEPT ? F / dF : div_nr(F, dF));
     if (!(pn > plow)) pn = 0.5 * (p + plow);
     conv = !st && fabs(pn - p) <= kNewtonTol * fabs(pn);
     p_last = p;
@@ -650,8 +787,8 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
   if (st) return st;
   if (conv && isfinite(wL.df) && isfinite(wR.df)) {
     double rL, dL, rR, dR;
-    star_density(qL, L, p_last, wL, rL, dL);
-    star_density(qR, Rs, p_last, wR, rR, dR);
+    star_density<KEPT>(qL, L, p_last, wL, rL, dL);
+    star_density<KEPT>(qR, Rs, p_last, wR, rR, dR);
     if (isfinite(dL) && isfinite(dR)) {
       const double d = p - p_last;
       out.p = p;
@@ -662,7 +799,7 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
       return M2C_OK;
     }
   }
-  return riemann_finish(qL, L, qR, Rs, plow, vacuum_test, conv, p, out, iters = it);
+  return riemann_finish<KEPT>(qL, L, qR, Rs, plow, vacuum_test, conv, p, out, iters = it);
 }
 
 // ---------------------------------------------------------------------------
@@ -850,6 +987,7 @@ static __device__ __noinline__ bool riemann_newton_f(const EosP<float>& qL, floa
   return false;
 }
 
+template <bool KEPT>
 static __device__ __noinline__ int riemann_solve_mixed(const EosP<float>& qLf, const EosDev& qL, double rl, double ul, double pl,
                                           const EosP<float>& qRf, const EosDev& qR, double rr, double ur, double pr,
                                           RiemannOut& out, int& iters,
@@ -858,16 +996,16 @@ static __device__ __noinline__ int riemann_solve_mixed(const EosP<float>& qLf, c
   int it32 = 0;
   Side L, Rs;
   if (riemann_newton_f(qLf, d2f(rl), d2f(ul), d2f(pl), qRf, d2f(rr), d2f(ur), d2f(pr), p32, it32, (float)p_start) &&
-      make_side(qL, rl, ul, pl, L) && make_side(qR, rr, ur, pr, Rs)) {
+      make_side<KEPT>(qL, rl, ul, pl, L) && make_side<KEPT>(qR, rr, ur, pr, Rs)) {
     const double plow = fmax(eos_plow(qL), eos_plow(qR));
     fix_substeps(qL, L, qR, Rs, plow);
     double p = f2d(p32);
     for (int k = 0; k < 2; ++k) {
       Wave wL, wR;
       double rL, dL, rR, dR;
-      if (!(p > plow) || wave(qL, L, p, wL) || wave(qR, Rs, p, wR)) break;
-      star_density(qL, L, p, wL, rL, dL);
-      star_density(qR, Rs, p, wR, rR, dR);
+      if (!(p > plow) || wave<KEPT>(qL, L, p, wL) || wave<KEPT>(qR, Rs, p, wR)) break;
+      star_density<KEPT>(qL, L, p, wL, rL, dL);
+      star_density<KEPT>(qR, Rs, p, wR, rR, dR);
       const double F = wL.f + wR.f + (Rs.u - L.u), dF = wL.df + wR.df;
       const double dp = -F / dF;
       // a slope that is not finite (a wave of rounding-level strength on a
@@ -886,7 +1024,7 @@ static __device__ __noinline__ int riemann_solve_mixed(const EosP<float>& qLf, c
       p += dp;
     }
   }
-  return riemann_solve(qL, rl, ul, pl, qR, rr, ur, pr, out, iters, p_start);
+  return riemann_solve<KEPT>(qL, rl, ul, pl, qR, rr, ur, pr, out, iters, p_start);
 }
 
 }  // namespace m2c

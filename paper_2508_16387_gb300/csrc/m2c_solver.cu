@@ -91,7 +91,6 @@ __global__ void __launch_bounds__(kFiverThreads, 1) k_fiver(const Grid* __restri
   const int slot = list_slot(mode);
   const int n = min(ctrl->nface[slot], G.face_cap);
   const double* __restrict__ Ws = stage_W(G, mode);
-  const long long N = G.N;
   const int per = min(kFiverThreads, max(1, (int)(((long long)n * gridDim.y + units - 1) / units)));
   if ((int)threadIdx.x >= per) return;
   for (int i = blockIdx.x * per + threadIdx.x; i < n; i += gridDim.x * per) {
@@ -104,8 +103,8 @@ __global__ void __launch_bounds__(kFiverThreads, 1) k_fiver(const Grid* __restri
     const EosDev& qa = G.eos[ia];
     const EosDev& qb = G.eos[ib];
     double Pa[5], Pb[5];
-    bool ok = cons_to_prim<double, true>(qa, qa, Ws, N, ca, Pa);
-    ok = cons_to_prim<double, true>(qb, qb, Ws, N, cb, Pb) && ok;
+    bool ok = cell_prims(G, ia, Ws, ca, Pa);
+    ok = cell_prims(G, ib, Ws, cb, Pb) && ok;
     double Fa[5] = {0, 0, 0, 0, 0}, Fb[5] = {0, 0, 0, 0, 0};
     RiemannOut rs;
     int its = 0;
@@ -128,10 +127,13 @@ __global__ void __launch_bounds__(kFiverThreads, 1) k_fiver(const Grid* __restri
       const double* P1 = mirror ? Pa : Pb;
       const double sgn = mirror ? -1.0 : 1.0;
       if (G.prec == M2C_MIXED && G.riemann_fp32_start)
-        st = riemann_solve_mixed(G.eosf[mirror ? ib : ia], q0, P0[0], sgn * P0[1 + d], P0[4], G.eosf[mirror ? ia : ib], q1,
-                                 P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start);
+        st = riemann_solve_mixed<true>(G.eosf[mirror ? ib : ia], q0, P0[0], sgn * P0[1 + d], P0[4], G.eosf[mirror ? ia : ib], q1,
+                                       P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start);
+      else if (G.prec == M2C_MIXED)
+        st = riemann_solve<true>(q0, P0[0], sgn * P0[1 + d], P0[4], q1, P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start);
       else
-        st = riemann_solve(q0, P0[0], sgn * P0[1 + d], P0[4], q1, P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start, true);
+        st = riemann_solve<false>(q0, P0[0], sgn * P0[1 + d], P0[4], q1, P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start,
+                                  true);
       if (pst && st == M2C_OK) *pst = rs.p;
       if (mirror) {
         const double r = rs.rhoL;
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(128) k_finish(const Grid* __restrict__ grids, 
       const double* __restrict__ Ws = stage_W(G, mode);
       const int m = G.id[c] & 1;
       double P[5];
-      if (!cons_to_prim<double, true>(G.eos[m], G.eos[m], Ws, N, c, P)) latch_error(ctrl, M2C_ENONPHYS, c);
+      if (!cell_prims(G, m, Ws, c, P)) latch_error(ctrl, M2C_ENONPHYS, c);
       const double r = G.x0 + ((double)(c % G.nx) + 0.5) * G.h;
       const double a = (G.geom == M2C_GEOM_SPHERICAL ? 2.0 : 1.0) / r * P[1];
 #pragma unroll
@@ -387,7 +389,6 @@ __global__ void __launch_bounds__(128) k_phase_fix(const Grid* __restrict__ grid
     const long long c = G.flips[t];
     const int i = (int)(c % G.nx), j = (int)((c / G.nx) % G.ny), k = (int)(c / ((long long)G.nx * G.ny));
     const int m = (G.id[c] >> 2) & 1;  // material at the end of the step
-    const EosDev& q = G.eos[m];
     double sum[5] = {0, 0, 0, 0, 0};
     int cnt = 0;
     // a neighbour position across a symmetry side is the mirror image of a cell
@@ -398,7 +399,7 @@ __global__ void __launch_bounds__(128) k_phase_fix(const Grid* __restrict__ grid
       const int new_id = (G.id[nb] >> 2) & 1;
       if (old_id == m && new_id == m) {
         double P[5];
-        if (!cons_to_prim<double, true>(q, q, G.W, N, nb, P)) latch_error(ctrl, M2C_ENONPHYS, nb);
+        if (!cell_prims(G, m, G.W, nb, P)) latch_error(ctrl, M2C_ENONPHYS, nb);
         if (mirrored(ii, G.nx, G.bc[0], G.bc[1])) P[1] = -P[1];
         if (mirrored(jj, G.ny, G.bc[2], G.bc[3])) P[2] = -P[2];
         if (mirrored(kk, G.nz, G.bc[4], G.bc[5])) P[3] = -P[3];
@@ -432,8 +433,8 @@ __global__ void __launch_bounds__(128) k_phase_fix(const Grid* __restrict__ grid
     double P[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) P[v] = sum[v] / cnt;
-    double e, c2;
-    if (!eos_e_c2<double, true>(q, P[0], 1.0 / P[0], P[4], e, c2)) latch_error(ctrl, M2C_ENONPHYS, c);
+    double e = 0.0;
+    if (!cell_energy(G, m, P[0], P[4], e)) latch_error(ctrl, M2C_ENONPHYS, c);
     G.W[c] = P[0];
     G.W[N + c] = P[0] * P[1];
     G.W[2 * N + c] = P[0] * P[2];
@@ -490,7 +491,7 @@ __global__ void k_state_to_prims(const Grid* __restrict__ grids, double* __restr
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
     const int m = lt0(G.phi[c]) ? 1 : 0;
     double P[5];
-    if (!cons_to_prim<double, true>(G.eos[m], G.eos[m], G.W, N, c, P)) latch_error(G.ctrl, M2C_ENONPHYS, c);
+    if (!cell_prims(G, m, G.W, c, P)) latch_error(G.ctrl, M2C_ENONPHYS, c);
 #pragma unroll
     for (int v = 0; v < 5; ++v) prims[v * N + c] = P[v];
   }
@@ -502,8 +503,8 @@ __global__ void k_prims_to_state(const Grid* __restrict__ grids, const double* _
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
     const int m = lt0(G.phi[c]) ? 1 : 0;
     const double rho = prims[c], u = prims[N + c], v = prims[2 * N + c], w = prims[3 * N + c], p = prims[4 * N + c];
-    double e, c2;
-    if (!eos_e_c2<double, true>(G.eos[m], rho, 1.0 / rho, p, e, c2)) latch_error(G.ctrl, M2C_ENONPHYS, c);
+    double e = 0.0;
+    if (!cell_energy(G, m, rho, p, e)) latch_error(G.ctrl, M2C_ENONPHYS, c);
     G.W[c] = rho;
     G.W[N + c] = rho * u;
     G.W[2 * N + c] = rho * v;
@@ -519,9 +520,9 @@ __global__ void k_riemann_batch(int n, EosDev qL, const double* __restrict__ L, 
     RiemannOut o;
     int its = 0;
     const int st =
-        mixed ? riemann_solve_mixed(qLf, qL, L[i], L[n + i], L[2 * n + i], qRf, qR, Rr[i], Rr[n + i], Rr[2 * n + i], o,
-                                    its)
-              : riemann_solve(qL, L[i], L[n + i], L[2 * n + i], qR, Rr[i], Rr[n + i], Rr[2 * n + i], o, its);
+        mixed ? riemann_solve_mixed<false>(qLf, qL, L[i], L[n + i], L[2 * n + i], qRf, qR, Rr[i], Rr[n + i],
+                                           Rr[2 * n + i], o, its)
+              : riemann_solve<false>(qL, L[i], L[n + i], L[2 * n + i], qR, Rr[i], Rr[n + i], Rr[2 * n + i], o, its);
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     out[i] = st ? nan : o.p;
     out[n + i] = st ? nan : o.u;
@@ -535,16 +536,16 @@ __global__ void k_riemann_batch(int n, EosDev qL, const double* __restrict__ L, 
 // Post-shock state from the right-facing wave curve of the Riemann solver.
 __global__ void k_shock_state(EosDev q, double rho, double u, double p, double p1, double* out, int* status) {
   Side K;
-  if (!make_side(q, rho, u, p, K) || !(p1 > p)) {
+  if (!make_side<true>(q, rho, u, p, K) || !(p1 > p)) {
     *status = M2C_EINVAL;
     return;
   }
   Wave w;
   double rs, drs;
-  const int st = wave(q, K, p1, w);
+  const int st = wave<true>(q, K, p1, w);
   *status = st;
   if (st) return;
-  star_density(q, K, p1, w, rs, drs);
+  star_density<true>(q, K, p1, w, rs, drs);
   out[0] = rs;
   out[1] = K.u + w.f;
   out[2] = (rs * out[1] - K.rho * K.u) / (rs - K.rho);
