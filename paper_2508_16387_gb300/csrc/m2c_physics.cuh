@@ -31,7 +31,7 @@ struct EosP {
   R rho0, c0, s, G0, e0, eta_min;            // MG
   R K0, rg, inv_rg, inv_2rho0, eta_max, pmin, rk4_span;  // MG derived
   R gm, ex, two_gm1, inv_g;                  // SG: (g-1)/(g+1), (g-1)/(2g), 2/(g-1), 1/g (Riemann wave curves)
-  R rmax, sG, gk, kap, kap2, rK;             // MG: rho0 s/(s-1), s - G0, G0/K0, (K0 rho0)^-1/2, 1/(K0 rho0), K0 rho0
+  R rmax, sG, gk, kap, kap2, rK;             // MG: rho0 s/(s-1), s - G0, G0/K0, (K0 rho0)^-1/2, 1/K0, K0 rho0
   R b, ec;                                   // NASG
   R om, A1, A2, R1r, R2r, c1, c2;            // JWL: w, A_i, R_i rho0, w/(R_i rho0)
 };
@@ -87,7 +87,7 @@ __host__ inline EosP<R> make_eos(int type, const double* prm) {
     e.rmax = (R)(prm[0] * prm[2] / (prm[2] - 1.0));
     e.sG = (R)(prm[2] - prm[3]);
     e.gk = (R)(prm[3] / K0);
-    e.kap2 = (R)(1.0 / (K0 * prm[0]));
+    e.kap2 = (R)(1.0 / K0);
     e.rK = (R)(K0 * prm[0]);
     e.kap = (R)sqrt(1.0 / (K0 * prm[0]));
   }

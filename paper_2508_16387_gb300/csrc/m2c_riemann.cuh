@@ -40,12 +40,12 @@ struct Side {
   // MG: 1/rho, 1/c^2; last Hugoniot root and its slope at pressure hp (NaN: none)
   double iv, ic2, hp, hr, hd;
   int nrk;  // RK4 substeps of this side's MG rarefaction curve in one problem; 0: per evaluation
-  // MG: spacing of the problem's fixed RK4 nodes p_K - i dnode (0: none), and the
-  // isentrope states (rho, f) after the first mbase and mbase - 1 full substeps, kept
-  // between the evaluations of one problem (nearby pressures share their nodes; the
-  // iteration may step back over one)
+  // MG: the density the isentrope starts from (rho, or rho/rho0: mg_rhs), the spacing of
+  // the problem's fixed RK4 nodes p_K - i dnode (0: none), and the isentrope states after
+  // the first mbase and mbase - 1 full substeps, kept between the evaluations of one
+  // problem (nearby pressures share their nodes; the iteration may step back over one)
   int mbase;
-  double dnode, idnode, dspan, rbase, fbase, rprev, fprev;  // dspan = nrk dnode, the span bound the nodes cover
+  double r0, dnode, idnode, dspan, rbase, fbase, rprev, fprev;  // dspan = nrk dnode, the span bound the nodes cover
 };
 
 template <bool KEPT>
@@ -84,7 +84,8 @@ __device__ inline bool make_side(const EosDev& q, double rho, double u, double p
     K.mbase = 0;
     K.dnode = 0.0;
     K.dspan = 0.0;
-    K.rbase = K.rprev = rho;
+    K.r0 = KEPT ? rho : rho * (2.0 * q.inv_2rho0);
+    K.rbase = K.rprev = K.r0;
     K.fbase = K.fprev = 0.0;
   }
   return true;
@@ -261,28 +262,30 @@ __device__ inline int mg_hugoniot(const EosDev& q, Side& K, double p, double& rh
   return st;
 }
 
-// Right-hand side of the MG isentrope. With d = rho - rho0 and q = rho - s d
-// (1 - s eta = q/rho) the sound speed of the compression branch is
-//   rho^2 c^2 = K0 rho0 A,  A = n rho^2/q^3 + g,  n = rho + (s - G0) d,  g = (G0/K0) p,
-// and the tension branch has the same form with q = rho (s = 0). d rho/dp = 1/c^2 =
-// (rho y)^2/(K0 rho0) and df/dp = 1/(rho c) = y/(K0 rho0)^(1/2) with y = A^(-1/2) =
-// q^2 (q (n rho^2 + g q^3))^(-1/2): 16 FP64 instructions with one root and no
+// Right-hand side of the MG isentrope in r = rho/rho0. With d = r - 1 and q = r - s d
+// (1 - s eta = q/r) the sound speed of the compression branch is
+//   rho^2 c^2 = K0 rho0 A,  A = n r^2/q^3 + g,  n = r + (s - G0) d,  g = (G0/K0) p,
+// and the tension branch has the same form with q = r (s = 0). dr/dp = 1/(rho0 c^2) =
+// (r y)^2/K0 and df/dp = 1/(rho c) = y/(K0 rho0)^(1/2) with y = A^(-1/2) =
+// q^2 (q (n r^2 + g q^3))^(-1/2): 16 FP64 instructions with one root and no
 // division (35 through the general e and c^2); the constant factors sit in the
-// substep lengths. ok is cleared outside the EOS domain (rho <= 0, eta >= 1/s,
-// c^2 <= 0). Below a finite tension cutoff A = g - (G0/K0) p_min.
-__device__ inline void mg_rhs(const EosDev& q, double g, double rho, double& kr, double& y, bool& ok) {
-  const double d = rho - q.rho0;
+// substep lengths, and r is of order 1 whatever the units of the density (in rho itself the
+// root's argument is of order rho^4, which left its range below 4e-10). ok is cleared
+// outside the EOS domain (rho <= 0, eta >= 1/s, c^2 not positive and finite). Below a
+// finite tension cutoff A = g - (G0/K0) p_min.
+__device__ inline void mg_rhs(const EosDev& q, double g, double r, double& kr, double& y, bool& ok) {
+  const double d = r - 1.0;
   const bool comp = gt0(d);
-  double qq = fma(comp ? -q.s : 0.0, d, rho);
-  const double n = fma(comp ? q.sG : -q.G0, d, rho);
-  double C = qq * fma(n, rho * rho, g * (qq * qq * qq)), q2 = qq * qq;
-  if (q.eta_min > -INFINITY && q.rho0 * rcp_nr(rho) > 1.0 - q.eta_min) {
+  double qq = fma(comp ? -q.s : 0.0, d, r);
+  const double n = fma(comp ? q.sG : -q.G0, d, r);
+  double C = qq * fma(n, r * r, g * (qq * qq * qq)), q2 = qq * qq;
+  if (q.eta_min > -INFINITY && rcp_nr(r) > 1.0 - q.eta_min) {
     C = g - q.gk * q.pmin;
     q2 = 1.0;
   }
-  ok = ok && gt0(rho) && gt0(qq) && nr_range_pos(C);
-  y = q2 * rsqrt_nr_in_range(C);
-  const double ry = rho * y;
+  ok = ok && gt0(r) && gt0(qq) && gt0(C) && hi_of(C) < 0x7ff00000u;
+  y = q2 * rsqrt_nr(C);
+  const double ry = r * y;
   kr = ry * ry;
 }
 
@@ -308,16 +311,16 @@ __device__ inline void mg_rk4_substep_kept(const EosDev& q, double pi, double hs
   fv = fv + h6 * (k1f + 2.0 * k2f + 2.0 * k3f + k4f);
 }
 
-// One classical RK4 substep of the MG isentrope (rho, f) from pressure pi by hs.
-__device__ inline void mg_rk4_substep(const EosDev& q, double pi, double hs, double& rho, double& fv, bool& ok) {
+// One classical RK4 substep of the MG isentrope (r, f) from pressure pi by hs.
+__device__ inline void mg_rk4_substep(const EosDev& q, double pi, double hs, double& r, double& fv, bool& ok) {
   const double g0 = q.gk * pi, gh = q.gk * hs, gm = fma(0.5, gh, g0);
   const double hr = hs * q.kap2, h2 = 0.5 * hr;
   double k1, k2, k3, k4, y1, y2, y3, y4;
-  mg_rhs(q, g0, rho, k1, y1, ok);
-  mg_rhs(q, gm, fma(h2, k1, rho), k2, y2, ok);
-  mg_rhs(q, gm, fma(h2, k2, rho), k3, y3, ok);
-  mg_rhs(q, g0 + gh, fma(hr, k3, rho), k4, y4, ok);
-  rho = fma(hr * (1.0 / 6.0), fma(2.0, k2 + k3, k1 + k4), rho);
+  mg_rhs(q, g0, r, k1, y1, ok);
+  mg_rhs(q, gm, fma(h2, k1, r), k2, y2, ok);
+  mg_rhs(q, gm, fma(h2, k2, r), k3, y3, ok);
+  mg_rhs(q, g0 + gh, fma(hr, k3, r), k4, y4, ok);
+  r = fma(hr * (1.0 / 6.0), fma(2.0, k2 + k3, k1 + k4), r);
   fv = fma(hs * (q.kap * (1.0 / 6.0)), fma(2.0, y2 + y3, y1 + y4), fv);
 }
 
@@ -361,7 +364,8 @@ __device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
     const double dp = __dsub_rn(K.p, p);
     // (kept: beyond the bound itself, equal substeps)
     const bool within = K.nrk > 1 && K.dnode > 0.0 && dp < (KEPT ? K.dspan : K.dspan + K.dnode);
-    double rho = K.rho, fv = 0.0, gap = 0.0, last = dp;
+    // (the isentrope's density: kept rho, else rho/rho0)
+    double rho = K.r0, fv = 0.0, gap = 0.0, last = dp;
     int i = 0, m = 0;
     if (within) {
       if constexpr (KEPT) {
@@ -429,8 +433,8 @@ __device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
       mg_rhs(q, q.gk * p, rho, k, y, ok);
       w.f = fv;
       w.df = y * q.kap;
-      w.a = rho;
-      w.b = k * q.kap2;
+      w.a = rho * q.rho0;
+      w.b = k * q.kap2 * q.rho0;
     }
     if (!ok) st = M2C_ENONPHYS;
   }

@@ -1,0 +1,45 @@
+"""The exact Riemann solver in other units, and at the edges of its equations of state."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2508_16387_gb300 import workloads as WL
+
+from test_gpu_parity import m2c  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def solve(M, eL, L, eR, R, **kw):
+    import torch
+    out, it, st = M.m2c_solve_riemann(eL, torch.from_numpy(L).cuda(), eR, torch.from_numpy(R).cuda(), **kw)
+    return out.cpu().numpy(), st.cpu().numpy()
+
+
+def mild_and_strong(n=3000):
+    rng = np.random.default_rng(5)
+    strong = rng.random(n) < 0.5
+    L = np.stack([rng.uniform(980, 1150, n), rng.uniform(-150, 300, n),
+                  np.where(strong, rng.uniform(1e8, 2e9, n), rng.uniform(9e4, 1e6, n))])
+    R = np.stack([rng.uniform(0.8, 6.0, n), rng.uniform(-50, 50, n), rng.uniform(8e4, 5e6, n)])
+    return L, R
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("k,m", [(-50, 0), (-34, -8), (40, 3)])
+def test_mie_grueneisen_in_other_units(m2c, k, m, mixed):  # noqa: F811
+    """Densities times 2^k, velocities times 2^m, pressures times 2^(k + 2m): the scaling is exact,
+    and the result scales with it. Only the roots and reciprocals whose operands leave the seeds'
+    range round differently; 1e-12 allows each of some thousand roundings of a curve one unit."""
+    L, R = mild_and_strong()
+    rho0, c0, s, g0 = WL.WATER_MG[1][:4]
+    ref, rst = solve(m2c, WL.WATER_MG, L, WL.AIR_PG, R, mixed=mixed)
+    scale = np.array([2.0 ** k, 2.0 ** m, 2.0 ** (k + 2 * m)])[:, None]
+    water = (WL.WATER_MG[0], (rho0 * 2.0 ** k, c0 * 2.0 ** m, s, g0))
+    out, st = solve(m2c, water, L * scale, WL.AIR_PG, R * scale, mixed=mixed)
+    assert np.array_equal(st, rst) and (rst == 0).mean() > 0.99
+    ok = rst == 0
+    back = np.array([2.0 ** (k + 2 * m), 2.0 ** m, 2.0 ** k, 2.0 ** k])[:, None]
+    for v in range(4):
+        scale_v = np.maximum(np.abs(ref[v][ok]), 150.0 if v == 1 else 0.0)
+        assert np.max(np.abs(out[v][ok] / back[v] - ref[v][ok]) / scale_v) < 1e-12, v
