@@ -605,9 +605,10 @@ __device__ inline void star_density(const EosDev& q, const Side& K, double p, co
     rs = K.rho * (r + q.gm) * id;
     drs = K.rho * fma(-q.gm, q.gm, 1.0) * (id * id) * K.ipb;
   } else {
-    // r^(1/g) = r/(r^((g-1)/(2g)))^2
-    const double pb = p + q.pc;
-    rs = K.rho * (pb * K.ipb) * rcp_nr(w.a * w.a);
+    // r^(1/g) = r/(r^((g-1)/(2g)))^2, r the IEEE quotient as in wave_sg: at p = p_K the
+    // density is the side's own to the bit (a contact stays one)
+    const double pb = p + q.pc, r0 = pb * K.ipb, r = fma(fma(-K.pb, r0, pb), K.ipb, r0);
+    rs = K.rho * r * rcp_nr(w.a * w.a);
     drs = rs * q.inv_g * rcp_nr(pb);
   }
 }

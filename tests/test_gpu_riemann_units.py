@@ -2,7 +2,6 @@
 import numpy as np
 import pytest
 
-from oracle import oracle as O
 from paper_2508_16387_gb300 import workloads as WL
 
 from test_gpu_parity import m2c  # noqa: F401
@@ -43,3 +42,16 @@ def test_mie_grueneisen_in_other_units(m2c, k, m, mixed):  # noqa: F811
     for v in range(4):
         scale_v = np.maximum(np.abs(ref[v][ok]), 150.0 if v == 1 else 0.0)
         assert np.max(np.abs(out[v][ok] / back[v] - ref[v][ok]) / scale_v) < 1e-12, v
+
+
+@pytest.mark.parametrize("water", [WL.WATER_SG, WL.WATER_MG], ids=["sg", "mg"])
+def test_a_contact_keeps_its_states(m2c, water):  # noqa: F811
+    """Equal pressures and velocities: no wave, and every value of the star states is its side's own."""
+    n = 4000
+    rng = np.random.default_rng(9)
+    p, u = rng.uniform(8e4, 5e6, n), rng.uniform(-100, 100, n)
+    L = np.stack([rng.uniform(990, 1100, n), u, p])
+    R = np.stack([rng.uniform(0.8, 6.0, n), u, p])
+    out, st = solve(m2c, water, L, WL.AIR_PG, R)
+    assert (st == 0).all()
+    assert np.array_equal(out, np.stack([p, u, L[0], R[0]]))
