@@ -759,12 +759,12 @@ int sm_count() {
 
 namespace {
 
-void set_tiling(Grid& g, int ty, int tz) {
+// requested: tz is the caller's own, else the automatic length.
+void set_tiling(Grid& g, int ty, int tz, bool requested) {
   g.tiles_x = (g.nx + 31) / 32;
   g.tiles_y = (g.ny + ty - 1) / ty;
-  g.tz = std::max(1, std::min(tz, g.nz));
+  g.tz = chunk_planes(g.nz, tz, requested);
   g.tiles_z = (g.nz + g.tz - 1) / g.tz;
-  g.tz = (g.nz + g.tiles_z - 1) / g.tiles_z;  // the same number of chunks, evenly
 }
 
 long long ntiles_of(const Grid& g) { return (long long)g.tiles_x * g.tiles_y * g.tiles_z; }
@@ -1078,7 +1078,7 @@ m2c_status m2c_init_grid(m2c_ctx** out, int nx, int ny, int nz, const double lo[
   c->stream = static_cast<cudaStream_t>(stream);
   setup_all_stage_kernels();
   c->ty = g.general ? 8 : default_rows(g);
-  set_tiling(g, c->ty, default_tz(g, c->ty));
+  set_tiling(g, c->ty, default_tz(g, c->ty), false);
   c->reinit_every = 10;
   c->reinit_iters = 5;
   g.reinit_every = 10;
@@ -1141,7 +1141,7 @@ static void update_general(m2c_ctx* c) {
                eos_extended(g.eos[1].type) || g.band_gamma > 0.0) ? 1 : 0;
   if (g.general && c->ty != 8) {
     c->ty = 8;
-    set_tiling(g, 8, default_tz(g, 8));
+    set_tiling(g, 8, default_tz(g, 8), false);
   }
 }
 
@@ -1194,7 +1194,7 @@ m2c_status m2c_set_tiling(m2c_ctx* c, int tile_rows, int tile_z) {
   if (c->host.general && tile_rows != 8)
     return set_err(c, M2C_EINVAL, "grids with scheme options run 8-row tiles");
   c->ty = tile_rows;
-  set_tiling(c->host, c->ty, tile_z > 0 ? tile_z : default_tz(c->host, c->ty));
+  set_tiling(c->host, c->ty, tile_z > 0 ? tile_z : default_tz(c->host, c->ty), tile_z > 0);
   return push_grid(c);
 }
 
@@ -1375,7 +1375,8 @@ m2c_status m2c_batch_create(m2c_batch** out, m2c_ctx** v, int k, void* workspace
                                                      align_up(sizeof(long long) * (size_t)(k + 1)));
   b->tiles.assign(k + 1, 0);
   b->nmax = 1;
-  if (tz <= 0) {
+  const bool tz_requested = tz > 0;
+  if (!tz_requested) {
     std::vector<const Grid*> gs;
     for (int i = 0; i < k; ++i) gs.push_back(&v[i]->host);
     tz = choose_tz(gs.data(), k, tile_shape(v[0]->host.prec, ty));
@@ -1384,7 +1385,7 @@ m2c_status m2c_batch_create(m2c_batch** out, m2c_ctx** v, int k, void* workspace
     m2c_ctx* c = v[order[i]];
     b->ctx.push_back(c);
     Grid g = c->host;
-    set_tiling(g, ty, tz);
+    set_tiling(g, ty, tz, tz_requested);
     b->hosts.push_back(g);
     b->tiles[i + 1] = b->tiles[i] + ntiles_of(g);
     b->nmax = std::max(b->nmax, g.N);
@@ -1776,7 +1777,7 @@ m2c_status m2c_residual_noalloc(int nx, int ny, int nz, double h, const int bc[6
   g.resR = R;
   g.resL = L;
   const int ty = 8;
-  set_tiling(g, ty, default_tz(g, ty));
+  set_tiling(g, ty, default_tz(g, ty), false);
   const long long tiles[2] = {0, ntiles_of(g)};
   Grid* dg = reinterpret_cast<Grid*>(ws + m2c::kNaGrid);
   long long* dt = reinterpret_cast<long long*>(ws + m2c::kNaTiles);

@@ -16,6 +16,15 @@ struct LaunchPlan {
   int mats = -1;         // EOS types of the two materials of every grid, T0 + 4 T1 (SG / MG); -1: mixed or other
 };
 
+// Planes of a tile's chunk along z on a grid of nz planes: a requested length is taken as
+// it is (at most nz); the automatic one is evened out over the same number of chunks.
+inline int chunk_planes(int nz, int tz, bool requested) {
+  tz = tz < 1 ? 1 : (tz < nz ? tz : nz);
+  if (requested) return tz;
+  const int chunks = (nz + tz - 1) / tz;
+  return (nz + chunks - 1) / chunks;
+}
+
 // Host-side state kept per device (index of the current device, clamped to
 // kMaxDevices - 1) and the current device's SM count.
 constexpr int kMaxDevices = 64;

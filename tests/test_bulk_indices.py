@@ -31,3 +31,9 @@ def test_cells_outside_a_tile_read_written_slots(tmp_path):
 def test_mapped_positions_are_cells_of_the_grid(tmp_path):
     """A position anywhere in a tile or its halo, however short the axis, maps to a cell of it."""
     assert "positions outside 0 wrong 0" in _run(tmp_path, "map_check")
+
+
+def test_requested_chunk_length_is_kept(tmp_path):
+    """The z-length a caller asks for (m2c_set_tiling, a batch's tuning) is the one that runs; only
+    the automatic one is evened out."""
+    assert "wrong chunks 0" in _run(tmp_path, "chunk_check")
