@@ -783,6 +783,15 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
     if (!st) st = sr;
     const double F = wL.f + wR.f + (Rs.u - L.u), dF = wL.df + wR.df;
     double pn = p - (KEPT ? F / dF : div_nr(F, dF));
+    if (isinf(dF)) {
+      // an iterate a few units above a side's pressure: its shock is too weak to resolve, and
+      // the slope of its curve infinite. The step F/F' = 0 says nothing then: the acoustic
+      // slope's step tells whether p is the root (a face at rest that starts from its own
+      // pressure) or only a start next to a side's pressure
+      const double dL = isinf(wL.df) ? 1.0 / (L.rho * L.c) : wL.df, dR = isinf(wR.df) ? 1.0 / (Rs.rho * Rs.c) : wR.df;
+      const double pa = p - F / (dL + dR);
+      if (!(fabs(pa - p) <= kNewtonTol * fabs(pa))) pn = pa;
+    }
     if (!(pn > plow)) pn = 0.5 * (p + plow);
     conv = !st && fabs(pn - p) <= kNewtonTol * fabs(pn);
     p_last = p;
