@@ -45,7 +45,8 @@ struct Side {
   // the first mbase and mbase - 1 full substeps, kept between the evaluations of one
   // problem (nearby pressures share their nodes; the iteration may step back over one)
   int mbase;
-  double r0, dnode, idnode, dspan, rbase, fbase, rprev, fprev;  // dspan = nrk dnode, the span bound the nodes cover
+  // dspan = nrk dnode, the span bound the nodes cover; dreach, how far iterates may use them
+  double r0, dnode, idnode, dspan, dreach, rbase, fbase, rprev, fprev;
 };
 
 template <bool KEPT>
@@ -64,6 +65,8 @@ __device__ inline bool make_side(const EosDev& q, double rho, double u, double p
   K.u = u;
   K.p = p;
   K.e = e;
+  K.nrk = 0;
+  K.dnode = K.dspan = K.dreach = 0.0;
   if (q.type == M2C_EOS_SG && KEPT) {
     K.pb = p + q.pc;
     K.z = rho * K.c;
@@ -80,10 +83,7 @@ __device__ inline bool make_side(const EosDev& q, double rho, double u, double p
     K.iv = iv;
     if constexpr (!KEPT) K.ic2 = rcp_nr(c2);
     K.hp = NAN;
-    K.nrk = 0;
     K.mbase = 0;
-    K.dnode = 0.0;
-    K.dspan = 0.0;
     K.r0 = KEPT ? rho : rho * (2.0 * q.inv_2rho0);
     K.rbase = K.rprev = K.r0;
     K.fbase = K.fprev = 0.0;
@@ -137,7 +137,7 @@ __device__ inline double fix_substeps(const EosDev& qL, Side& L, const EosDev& q
     K.nrk = mg_substeps(q, span);
     K.dnode = (span > 0.0 && isfinite(span)) ? div_nr(span, (double)K.nrk) : 0.0;
     K.idnode = rcp_nr(K.dnode);
-    K.dspan = __dmul_rn((double)K.nrk, K.dnode);
+    K.dspan = K.dreach = __dmul_rn((double)K.nrk, K.dnode);
   };
   if (qL.type == M2C_EOS_MG) mg_nodes(qL, L, loL);
   if (qR.type == M2C_EOS_MG) mg_nodes(qR, Rs, loR);
@@ -328,10 +328,12 @@ __device__ inline void mg_rk4_substep(const EosDev& q, double pi, double hs, dou
 // inside a problem's span bound on the fixed nodes p_K - i dnode (full substeps
 // down to the last node above p, resumed from a node reached by an earlier
 // evaluation of the problem, then one partial substep to p): the curve is
-// continuous and smooth in p. An iterate less than a node spacing beyond the bound
-// takes all nodes and the partial substep too (the root lies inside the bound, and
-// the nodes serve the next iterate); further beyond, and for a wave evaluated
-// alone, equal substeps over p_K - p. All are one loop, so that the lanes of a
+// continuous and smooth in p. Beyond the bound, and for a wave evaluated alone, equal
+// substeps over p_K - p. An iterate less than a node spacing beyond the bound may take all
+// nodes and the partial substep too (dreach: the nodes serve the next iterate; half the
+// time of a batch of water against air), but no solution does: an isentrope into strong
+// tension is not convex, its root can lie beyond the acoustic bound, and there the nodes
+// carried on were 1e-8 off the equal substeps. All are one loop, so that the lanes of a
 // warp take their substeps together. The node arithmetic is written without
 // contracted multiply-adds, so that it takes the same nodes as the oracle.
 template <bool KEPT>
@@ -362,8 +364,7 @@ __device__ inline int wave_mg(const EosDev& q, Side& K, double p, Wave& w) {
     w.b = drdp;
   } else {
     const double dp = __dsub_rn(K.p, p);
-    // (kept: beyond the bound itself, equal substeps)
-    const bool within = K.nrk > 1 && K.dnode > 0.0 && dp < (KEPT ? K.dspan : K.dspan + K.dnode);
+    const bool within = K.nrk > 1 && K.dnode > 0.0 && dp < K.dreach;
     // (the isentrope's density: kept rho, else rho/rho0)
     double rho = K.r0, fv = 0.0, gap = 0.0, last = dp;
     int i = 0, m = 0;
@@ -623,6 +624,12 @@ static __device__ __noinline__ int riemann_F(const EosDev& qL, Side& L, const Eo
   return st;
 }
 
+// Whether the MG isentrope of a side was evaluated at p on nodes beyond its span bound.
+__device__ inline bool on_nodes_beyond(const Side& K, double p) {
+  const double dp = __dsub_rn(K.p, p);
+  return K.nrk > 1 && dp >= K.dspan && dp < K.dreach;
+}
+
 struct RiemannOut {
   double p, u, rhoL, rhoR;
 };
@@ -769,13 +776,17 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
     if (!(gap > 0.0)) gap = fmax(L.p, Rs.p) - plow;
     p = plow + 1e-3 * gap;
   }
+  if constexpr (!KEPT) {
+    L.dreach = L.dspan + L.dnode;
+    Rs.dreach = Rs.dspan + Rs.dnode;
+  }
   // the solution follows from the last evaluation to first order in its step (at
   // most the tolerance: the error is of the order of its square) instead of from
   // one more evaluation
   Wave wL{}, wR{};
   double p_last = p;
   bool conv = false, more = true;
-  int it = 0;
+  int it = 0, counted = 0;
   while (more) {
     ++it;
     st = wave<KEPT>(qL, L, p, wL);
@@ -794,10 +805,22 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
     }
     if (!(pn > plow)) pn = 0.5 * (p + plow);
     conv = !st && fabs(pn - p) <= kNewtonTol * fabs(pn);
+    if constexpr (!KEPT) {
+      // a root found on nodes beyond a side's bound: on with the equal substeps (a step or
+      // two within 1e-8 of p, which the count leaves out: the oracle takes them from the start)
+      if (conv && (on_nodes_beyond(L, p) || on_nodes_beyond(Rs, p))) {
+        L.dreach = L.dspan;
+        Rs.dreach = Rs.dspan;
+        conv = false;
+        counted = it;
+      }
+    }
     p_last = p;
     p = pn;
     more = !st && !conv && it < kNewtonCap;
   }
+  L.dreach = L.dspan;
+  Rs.dreach = Rs.dspan;
   if (st) return st;
   if (conv && isfinite(wL.df) && isfinite(wR.df)) {
     double rL, dL, rR, dR;
@@ -809,7 +832,7 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
       out.u = 0.5 * (L.u + Rs.u) + 0.5 * (wR.f - wL.f) + 0.5 * (wR.df - wL.df) * d;
       out.rhoL = rL + dL * d;
       out.rhoR = rR + dR * d;
-      iters = it;
+      iters = counted ? counted : it;
       return M2C_OK;
     }
   }

@@ -2,6 +2,7 @@
 import numpy as np
 import pytest
 
+from oracle import oracle as O
 from paper_2508_16387_gb300 import workloads as WL
 
 from test_gpu_parity import m2c  # noqa: F401
@@ -55,3 +56,28 @@ def test_a_contact_keeps_its_states(m2c, water):  # noqa: F811
     out, st = solve(m2c, water, L, WL.AIR_PG, R)
     assert (st == 0).all()
     assert np.array_equal(out, np.stack([p, u, L[0], R[0]]))
+
+
+def wide(rng, lo, hi, n):
+    """Wide states of a condensed material: a third in tension, velocities from 1 to 1e4."""
+    p = np.where(rng.random(n) < 0.3, -rng.uniform(0, 3.6e8, n), np.exp(rng.uniform(np.log(1e3), np.log(1e10), n)))
+    return np.stack([rng.uniform(lo, hi, n), rng.uniform(-1, 1, n) * 10 ** rng.uniform(0, 4, n), p])
+
+
+def against_oracle(M, eL, L, eR, R):
+    """1e-9 of each value (u*: of at least 1), equal statuses."""
+    ref, _, rst = O.riemann_batch(O.EOS(*eL), L, O.EOS(*eR), R)
+    out, st = solve(M, eL, L, eR, R)
+    assert np.array_equal(st, rst)
+    ok = rst == 0
+    for v in range(4):
+        scale = np.maximum(np.abs(ref[v][ok]), 1.0 if v == 1 else 1e-300)
+        assert np.max(np.abs(out[v][ok] - ref[v][ok]) / scale) < 1e-9, v
+
+
+def test_roots_beyond_the_acoustic_bound(m2c):  # noqa: F811
+    """Water against copper, both without a tension cutoff, down to tensions of 1e10 Pa, where the
+    root can lie beyond the pressure span that the fixed nodes of the isentrope cover."""
+    rng = np.random.default_rng(17)
+    copper = (WL.WATER_MG[0], (8930.0, 3940.0, 1.489, 1.99))
+    against_oracle(m2c, WL.WATER_MG, wide(rng, 900, 1500, 20000), copper, wide(rng, 8000, 11000, 20000))
