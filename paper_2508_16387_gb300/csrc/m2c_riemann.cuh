@@ -19,7 +19,10 @@ namespace m2c {
 // KEPT (template parameter below): the arithmetic of a mixed grid's interface (rcp_kept in
 // m2c_physics.cuh says why it is kept), in the same control flow: IEEE roots and quotients,
 // two-step reciprocals, the general e and c^2 along the isentrope, the PVRS start. Without
-// it, the shorter forms of FP64 grids and Riemann batches. What it costs: a FIVER launch of
+// it, the shorter forms of FP64 grids and Riemann batches. Materials with a finite tension
+// cutoff take the kept arithmetic everywhere (has_cutoff): their isentrope can cross the jump
+// of c^2 at the cutoff, where last bits and the way the iterates come decide between two
+// roots, or whether one is found at all. What it costs: a FIVER launch of
 // a late shock-bubble takes 2300 us at 192^3 and 1270 at 131x67x45, against 980 and 312 with
 // the shorter forms (3188 and 1733 with the kept arithmetic before the control flow was made
 // reconvergent): 35 FP64 instructions instead of 16 in the isentrope's right-hand side, and
@@ -98,6 +101,9 @@ __device__ inline double eos_plow(const EosDev& q) {
   if (q.type == M2C_EOS_JWL) return 0.0;
   return isfinite(q.eta_min) ? q.pmin : -INFINITY;
 }
+
+// An MG material with a finite tension cutoff.
+__device__ inline bool has_cutoff(const EosDev& q) { return q.type == M2C_EOS_MG && q.eta_min > -INFINITY; }
 
 // Equal RK4 substeps over a pressure span dp of an MG isentrope: 64 for a span
 // of at least 5% of K0 = rho0 c0^2, proportionally fewer (at least one) below.
@@ -271,18 +277,14 @@ __device__ inline int mg_hugoniot(const EosDev& q, Side& K, double p, double& rh
 // division (35 through the general e and c^2); the constant factors sit in the
 // substep lengths, and r is of order 1 whatever the units of the density (in rho itself the
 // root's argument is of order rho^4, which left its range below 4e-10). ok is cleared
-// outside the EOS domain (rho <= 0, eta >= 1/s, c^2 not positive and finite). Below a
-// finite tension cutoff A = g - (G0/K0) p_min.
+// outside the EOS domain (rho <= 0, eta >= 1/s, c^2 not positive and finite). Materials with
+// a finite tension cutoff do not come here (has_cutoff).
 __device__ inline void mg_rhs(const EosDev& q, double g, double r, double& kr, double& y, bool& ok) {
   const double d = r - 1.0;
   const bool comp = gt0(d);
   double qq = fma(comp ? -q.s : 0.0, d, r);
   const double n = fma(comp ? q.sG : -q.G0, d, r);
-  double C = qq * fma(n, r * r, g * (qq * qq * qq)), q2 = qq * qq;
-  if (q.eta_min > -INFINITY && rcp_nr(r) > 1.0 - q.eta_min) {
-    C = g - q.gk * q.pmin;
-    q2 = 1.0;
-  }
+  const double C = qq * fma(n, r * r, g * (qq * qq * qq)), q2 = qq * qq;
   ok = ok && gt0(r) && gt0(qq) && gt0(C) && hi_of(C) < 0x7ff00000u;
   y = q2 * rsqrt_nr(C);
   const double ry = r * y;

@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kFiverThreads, 1) k_fiver(const Grid* __restri
       if (G.prec == M2C_MIXED && G.riemann_fp32_start)
         st = riemann_solve_mixed<true>(G.eosf[mirror ? ib : ia], q0, P0[0], sgn * P0[1 + d], P0[4], G.eosf[mirror ? ia : ib], q1,
                                        P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start);
-      else if (G.prec == M2C_MIXED)
+      else if (G.prec == M2C_MIXED || has_cutoff(qa) || has_cutoff(qb))
         st = riemann_solve<true>(q0, P0[0], sgn * P0[1 + d], P0[4], q1, P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start);
       else
         st = riemann_solve<false>(q0, P0[0], sgn * P0[1 + d], P0[4], q1, P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start,
@@ -519,10 +519,15 @@ __global__ void k_riemann_batch(int n, EosDev qL, const double* __restrict__ L, 
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     RiemannOut o;
     int its = 0;
-    const int st =
-        mixed ? riemann_solve_mixed<false>(qLf, qL, L[i], L[n + i], L[2 * n + i], qRf, qR, Rr[i], Rr[n + i],
-                                           Rr[2 * n + i], o, its)
-              : riemann_solve<false>(qL, L[i], L[n + i], L[2 * n + i], qR, Rr[i], Rr[n + i], Rr[2 * n + i], o, its);
+    const double rL = L[i], uL = L[n + i], pL = L[2 * n + i], rR = Rr[i], uR = Rr[n + i], pR = Rr[2 * n + i];
+    const bool kept = has_cutoff(qL) || has_cutoff(qR);
+    int st;
+    if (mixed)
+      st = kept ? riemann_solve_mixed<true>(qLf, qL, rL, uL, pL, qRf, qR, rR, uR, pR, o, its)
+                : riemann_solve_mixed<false>(qLf, qL, rL, uL, pL, qRf, qR, rR, uR, pR, o, its);
+    else
+      st = kept ? riemann_solve<true>(qL, rL, uL, pL, qR, rR, uR, pR, o, its)
+                : riemann_solve<false>(qL, rL, uL, pL, qR, rR, uR, pR, o, its);
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     out[i] = st ? nan : o.p;
     out[n + i] = st ? nan : o.u;

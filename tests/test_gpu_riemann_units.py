@@ -65,11 +65,14 @@ def wide(rng, lo, hi, n):
 
 
 def against_oracle(M, eL, L, eR, R):
-    """1e-9 of each value (u*: of at least 1), equal statuses."""
-    ref, _, rst = O.riemann_batch(O.EOS(*eL), L, O.EOS(*eR), R)
+    """Equal statuses; 1e-9 of each value (u*: of at least 1) where the oracle's Newton iteration
+    converges. A problem that it leaves to the bisection has the jump of a curve at its root: the
+    last bits decide which side of it is returned."""
+    ref, rit, rst = O.riemann_batch(O.EOS(*eL), L, O.EOS(*eR), R)
     out, st = solve(M, eL, L, eR, R)
     assert np.array_equal(st, rst)
-    ok = rst == 0
+    ok = (rst == 0) & (rit <= 50)
+    assert ok.sum() > 0.99 * (rst == 0).sum()
     for v in range(4):
         scale = np.maximum(np.abs(ref[v][ok]), 1.0 if v == 1 else 1e-300)
         assert np.max(np.abs(out[v][ok] - ref[v][ok]) / scale) < 1e-9, v
@@ -81,3 +84,19 @@ def test_roots_beyond_the_acoustic_bound(m2c):  # noqa: F811
     rng = np.random.default_rng(17)
     copper = (WL.WATER_MG[0], (8930.0, 3940.0, 1.489, 1.99))
     against_oracle(m2c, WL.WATER_MG, wide(rng, 900, 1500, 20000), copper, wide(rng, 8000, 11000, 20000))
+
+
+@pytest.mark.parametrize("other", ["water", "air"])
+def test_finite_tension_cutoff(m2c, other):  # noqa: F811
+    """Water with a tension cutoff at a strain of -0.02: the same problems are refused, and the roots
+    are the oracle's."""
+    rng = np.random.default_rng(3)
+    n = 20000
+    water = (WL.WATER_MG[0], (1000.0, 1483.0, 1.75, 0.28, 0.0, -0.02))
+    L = wide(rng, 800, 1500, n)
+    if other == "water":
+        against_oracle(m2c, water, L, water, wide(rng, 800, 1500, n))
+    else:
+        R = np.stack([np.exp(rng.uniform(np.log(0.01), np.log(100), n)), rng.uniform(-1, 1, n) * 10 ** rng.uniform(0, 4, n),
+                      np.exp(rng.uniform(np.log(10), np.log(1e8), n))])
+        against_oracle(m2c, water, L, WL.AIR_PG, R)
