@@ -798,12 +798,16 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
     double pn = p - (KEPT ? F / dF : div_nr(F, dF));
     if (isinf(dF)) {
       // an iterate a few units above a side's pressure: its shock is too weak to resolve, and
-      // the slope of its curve infinite. The step F/F' = 0 says nothing then: the acoustic
-      // slope's step tells whether p is the root (a face at rest that starts from its own
-      // pressure) or only a start next to a side's pressure
-      const double dL = isinf(wL.df) ? 1.0 / (L.rho * L.c) : wL.df, dR = isinf(wR.df) ? 1.0 / (Rs.rho * Rs.c) : wR.df;
-      const double pa = p - F / (dL + dR);
-      if (!(fabs(pa - p) <= kNewtonTol * fabs(pa))) pn = pa;
+      // the slope of its curve infinite. The step F/F' = 0 says nothing then: the step with
+      // that side's acoustic curve tells whether p is the root (a face at rest that starts
+      // from its own pressure; to the tolerance, or to the last bit of rho c^2, which is what
+      // a curve resolves) or only a start next to a side's pressure
+      const bool iL = isinf(wL.df), iR = isinf(wR.df);
+      const double dL = iL ? 1.0 / (L.rho * L.c) : wL.df, dR = iR ? 1.0 / (Rs.rho * Rs.c) : wR.df;
+      const double fL = iL ? (p - L.p) * dL : wL.f, fR = iR ? (p - Rs.p) * dR : wR.f;
+      const double pa = p - (fL + fR + (Rs.u - L.u)) / (dL + dR);
+      const double res = 0x1p-52 * fmax(iL ? L.rho * L.c * L.c : 0.0, iR ? Rs.rho * Rs.c * Rs.c : 0.0);
+      if (!(fabs(pa - p) <= fmax(kNewtonTol * fabs(pa), res))) pn = pa;
     }
     if (!(pn > plow)) pn = 0.5 * (p + plow);
     conv = !st && fabs(pn - p) <= kNewtonTol * fabs(pn);
