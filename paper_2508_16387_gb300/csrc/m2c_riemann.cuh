@@ -746,11 +746,13 @@ static __device__ __noinline__ double start_guess(const EosDev& qL, const Side& 
 // solve); NaN, or a value not above the lowest admissible pressure, takes the
 // PVRS estimate, or, with `guess`, start_guess() where the PVRS estimate and the
 // acoustic pressure differ by more than 5 %. The root and the stopping rule do
-// not depend on the start.
+// not depend on the start. resolution: of a pressure, in units of rho c^2 (used where a
+// shock is too weak to resolve): the last bit of 64, which is what a curve resolves; on
+// mixed grids the binary32 unit 2^-24 of the strains that their pressures come from.
 template <bool KEPT>
 static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, double ul, double pl, const EosDev& qR, double rr,
                                     double ur, double pr, RiemannOut& out, int& iters,
-                                    double p_start = NAN, bool guess = false) {
+                                    double p_start = NAN, bool guess = false, double resolution = 0x1p-52) {
   Side L, Rs;
   iters = 0;
   if (!make_side<KEPT>(qL, rl, ul, pl, L) || !make_side<KEPT>(qR, rr, ur, pr, Rs)) return M2C_ENONPHYS;
@@ -800,13 +802,13 @@ static __device__ __noinline__ int riemann_solve(const EosDev& qL, double rl, do
       // an iterate a few units above a side's pressure: its shock is too weak to resolve, and
       // the slope of its curve infinite. The step F/F' = 0 says nothing then: the step with
       // that side's acoustic curve tells whether p is the root (a face at rest that starts
-      // from its own pressure; to the tolerance, or to the last bit of rho c^2, which is what
-      // a curve resolves) or only a start next to a side's pressure
+      // from its own pressure; to the tolerance, or to the resolution times rho c^2) or only a
+      // start next to a side's pressure
       const bool iL = isinf(wL.df), iR = isinf(wR.df);
       const double dL = iL ? 1.0 / (L.rho * L.c) : wL.df, dR = iR ? 1.0 / (Rs.rho * Rs.c) : wR.df;
       const double fL = iL ? (p - L.p) * dL : wL.f, fR = iR ? (p - Rs.p) * dR : wR.f;
       const double pa = p - (fL + fR + (Rs.u - L.u)) / (dL + dR);
-      const double res = 0x1p-52 * fmax(iL ? L.rho * L.c * L.c : 0.0, iR ? Rs.rho * Rs.c * Rs.c : 0.0);
+      const double res = resolution * fmax(iL ? L.rho * L.c * L.c : 0.0, iR ? Rs.rho * Rs.c * Rs.c : 0.0);
       if (!(fabs(pa - p) <= fmax(kNewtonTol * fabs(pa), res))) pn = pa;
     }
     if (!(pn > plow)) pn = 0.5 * (p + plow);
@@ -1034,7 +1036,7 @@ template <bool KEPT>
 static __device__ __noinline__ int riemann_solve_mixed(const EosP<float>& qLf, const EosDev& qL, double rl, double ul, double pl,
                                           const EosP<float>& qRf, const EosDev& qR, double rr, double ur, double pr,
                                           RiemannOut& out, int& iters,
-                                          double p_start = NAN) {
+                                          double p_start = NAN, double resolution = 0x1p-52) {
   float p32;
   int it32 = 0;
   Side L, Rs;
@@ -1067,7 +1069,7 @@ static __device__ __noinline__ int riemann_solve_mixed(const EosP<float>& qLf, c
       p += dp;
     }
   }
-  return riemann_solve<KEPT>(qL, rl, ul, pl, qR, rr, ur, pr, out, iters, p_start);
+  return riemann_solve<KEPT>(qL, rl, ul, pl, qR, rr, ur, pr, out, iters, p_start, false, resolution);
 }
 
 }  // namespace m2c

@@ -128,9 +128,10 @@ __global__ void __launch_bounds__(kFiverThreads, 1) k_fiver(const Grid* __restri
       const double sgn = mirror ? -1.0 : 1.0;
       if (G.prec == M2C_MIXED && G.riemann_fp32_start)
         st = riemann_solve_mixed<true>(G.eosf[mirror ? ib : ia], q0, P0[0], sgn * P0[1 + d], P0[4], G.eosf[mirror ? ia : ib], q1,
-                                       P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start);
+                                       P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start, 0x1p-24);
       else if (G.prec == M2C_MIXED || has_cutoff(qa) || has_cutoff(qb))
-        st = riemann_solve<true>(q0, P0[0], sgn * P0[1 + d], P0[4], q1, P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start);
+        st = riemann_solve<true>(q0, P0[0], sgn * P0[1 + d], P0[4], q1, P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start,
+                                 false, G.prec == M2C_MIXED ? 0x1p-24 : 0x1p-52);
       else
         st = riemann_solve<false>(q0, P0[0], sgn * P0[1 + d], P0[4], q1, P1[0], sgn * P1[1 + d], P1[4], rs, its, p_start,
                                   true);

@@ -37,3 +37,27 @@ def test_faces_leaving_rest_match_oracle(m2c, p0):  # noqa: F811
         g.step(3)
         g.sync()
         assert max(rel_err(g.W.cpu().numpy(), ref.W)) <= tol, prec
+
+
+def test_a_repeated_host_pass_repeats_its_result(m2c):  # noqa: F811
+    """upload, ten steps, download three times on the same host state (the second time with another
+    state in between): the faces' star pressures of an earlier pass only start the iteration. FP64
+    1e-12 of the largest value: ten steps of a run whose roots agree to the iteration's tolerance."""
+    import torch
+    from test_gpu_mixed_bits import AIR, MG, state
+    n = (45, 38, 33)
+    h, W, phi = state(n, MG, False)
+    g = m2c.Grid(n, h, (0,) * 6, (MG, AIR))
+    g.set_state()
+    W, phi = torch.from_numpy(W).contiguous().pin_memory(), torch.from_numpy(phi).contiguous().pin_memory()
+    other = (W.flip(3).contiguous().pin_memory(), phi.flip(2).contiguous().pin_memory())
+    other[0][1].neg_()
+    out = []
+    for src in ((W, phi), other, (W, phi)):
+        res = (torch.empty_like(W).pin_memory(), torch.empty_like(phi).pin_memory())
+        g.upload(*src)
+        g.step(10)
+        g.download(*res)
+        g.sync()
+        out.append(res[0].numpy())
+    assert max(rel_err(out[2], out[0])) <= 1e-12
