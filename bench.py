@@ -330,10 +330,9 @@ def _kernel_source_hash():
     return h.hexdigest()[:16]
 
 
-def _ncu_per_launch(key, n):
-    """A per-launch counter of the bulk stage kernel from the committed ncu summary, scaled from
-    256^3 to n^3 (both grow with the cells); None if the kernel sources changed since the
-    counters were taken."""
+def _ncu_value(key):
+    """A counter of the bulk stage kernel from the committed ncu summary; None if the kernel
+    sources changed since the counters were taken."""
     path = os.path.join(ROOT, "profiles", "stage_kernel_traffic.txt")
     try:
         vals = {}
@@ -344,9 +343,15 @@ def _ncu_per_launch(key, n):
                     vals[k.strip()] = v.strip()
         if vals.get("kernel_source_sha256_16") != _kernel_source_hash():
             return None
-        return float(vals[key]) * (n / 256.0) ** 3
+        return float(vals[key])
     except (OSError, KeyError, ValueError):
         return None
+
+
+def _ncu_per_launch(key, n):
+    """A per-launch counter, scaled from 256^3 to n^3 (they grow with the cells)."""
+    v = _ncu_value(key)
+    return None if v is None else v * (n / 256.0) ** 3
 
 
 def ncu_traffic(kind, n):
@@ -429,16 +434,15 @@ def run_ours(args):
     value = ws * N * args.steps / (t_max * 1e-3) / 1e6
     hbm, src = peaks()
     avg = kms / max(kl, 1)
-    # tile rows of the bulk kernel: the requested ones, else the library's default rule
+    # tile rows of the bulk kernel: the requested ones, else the mixed path's default
     sms = torch.cuda.get_device_properties(local).multi_processor_count
-    nx, ny, nz = s.n
-    rows = args.tile_rows or (16 if -(-nx // 32) * -(-ny // 16) * -(-nz // 16) >= 8 * sms else 8)
+    rows = args.tile_rows or 8
     alg_bytes = 120.0 * N  # mean over stage 1 (96 B/cell) and stage 2 (144 B/cell)
     achieved = alg_bytes / (avg * 1e-3) / 1e9
     roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
             "frac": round(achieved / hbm, 4), "traffic": ncu_traffic(args.prec, args.n),
             "kernel": f"k_stage<float,{rows}> (bulk stage)" if args.prec == "mixed"
-                      else "k_stage<double,8> (bulk stage)", "peak_source": src,
+                      else "k_stage<double> (bulk stage)", "peak_source": src,
             "kernel_ms_avg": round(avg, 4), "kernel_share": round(kms / ms, 3) if ms > 0 else None,
             "step_breakdown_ms": {k: round(v[0] / args.steps, 4) for k, v in time_steps.kernels.items()},
             "issue": issue_roofline(_ncu_per_launch(f"{args.prec}_warp_inst_per_launch_256", args.n), avg, sms,
@@ -483,7 +487,7 @@ def run_ours(args):
                              "flops_source": "op-counting build of the oracle (profiles/fp64_flops_per_cell_update.txt)"
                                              "; add, mul, div, sqrt one FLOP each; achieved over the whole step",
                              "peak_source": "measured 1.89 DFMA/clk/SM x 2 FLOPs x SMs x median sampled SM clock",
-                             "fp64_pipe_busy_ncu": 0.72, "kernel": "k_stage<double,8> (bulk stage)",
+                             "fp64_pipe_busy_ncu": _ncu_value("fp64_pipe_busy"), "kernel": "k_stage<double> (bulk stage)",
                              "kernel_ms_avg": round(avg64, 4), "traffic": ncu_traffic("fp64", args.n),
                              "hbm_frac": round(alg_bytes / (avg64 * 1e-3) / 1e9 / hbm, 4)}}
         del g64

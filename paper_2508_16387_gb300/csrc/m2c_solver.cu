@@ -791,10 +791,14 @@ m2c_status push_grid(m2c_ctx* c) {
 // locally uniform plane is cheaper). Estimated launch time in plane times of one
 // resident block: below one tile per slot the tiles run side by side, the most
 // loaded SM sets the time; above, the tiles' planes over the slots plus three
-// quarters of a tile of tail. slots = resident blocks x SMs; t1 and tR are the
+// quarters of a tile of tail. The tail and the factor 1.7 of a launch of one wave (nothing
+// fills the time between its shortest and its longest tile) are fitted to two launches,
+// 128^3 FP64 and a mixed batch, which other constants had slowed to 0.85 and 0.96 of the
+// fixed 16-plane chunks. slots = resident blocks x SMs; t1 and tR are the
 // times of a plane with one and with all `blocks` of them on the SM: a plane takes
 // 9 us alone and 13.5 us beside another in the mixed kernel (8 rows; latency
-// bound), and as long as the FP64 pipe needs in the FP64 kernel. Measured per
+// bound); the FP64 shapes are in planes of an 8-row tile, assumed and not measured apart:
+// 8 rows fill the FP64 pipe alone, two blocks of 4 rows take 5 % longer. Measured per
 // launch with fixed 16-plane chunks, and with this rule on the same kernel:
 // 48^3 mixed 242 -> 38 us, 131x67x45 mixed 381 -> 120, 112^3 mixed 281 -> 201,
 // 128x4x4 FP64 207 -> 55, 128^3 FP64 2795 -> 2664 (the present kernel: 48^3

@@ -163,9 +163,10 @@ __device__ __forceinline__ void material_faces(EA&& eos, int ic, const R Pm[5], 
 //
 // What bounds it: FP32 tiles the instruction issue and the latency of each warp's
 // chain (about 820 instructions a cell and stage without any face state, 1700 in an
-// early shock-bubble), compiled for 512 resident threads per SM (128 registers, no
-// spills; with 1024 threads at 64 registers the spills went to L2, the shared memory
-// leaving little L1, and took as long); FP64 tiles the FP64 pipe. Against face states
+// early shock-bubble), compiled for 512 resident threads per SM (128 registers; no
+// spills but 8 to 32 bytes in the MG/SG and SG/MG kernels of batches; with 1024 threads at
+// 64 registers the spills went to L2, the shared memory leaving little L1, and took as
+// long); FP64 tiles the FP64 pipe. Against face states
 // and fluxes as items distributed over the threads (2.2 and 2.1 a thread, all states
 // and fluxes through shared memory, three barriers, no uniform rows), per launch:
 // 256^3 mixed 1947 -> 1617 us, 192^3 with the shock in the bubble 1028 -> 927,
