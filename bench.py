@@ -485,7 +485,8 @@ def run_ours(args):
                              "frac": round(ach / peak64, 4) if ach else None,
                              "flops_per_cell_update": fpc,
                              "flops_source": "op-counting build of the oracle (profiles/fp64_flops_per_cell_update.txt)"
-                                             "; add, mul, div, sqrt one FLOP each; achieved over the whole step",
+                                             "; add, mul, div, sqrt one FLOP each; achieved over the whole step, every cell counted "
+                                             "(rows at rest or uniform take fewer, so the fraction can exceed 1)",
                              "peak_source": "measured 1.89 DFMA/clk/SM x 2 FLOPs x SMs x median sampled SM clock",
                              "fp64_pipe_busy_ncu": _ncu_value("fp64_pipe_busy"), "kernel": "k_stage<double> (bulk stage)",
                              "kernel_ms_avg": round(avg64, 4), "traffic": ncu_traffic("fp64", args.n),
