@@ -202,8 +202,8 @@ m2c_status m2c_set_riemann_start(m2c_ctx* ctx, int fp32_start);
 /* Tile of the bulk stage kernel: 32 x tile_rows (4 or 8; 16 for M2C_MIXED)
  * columns marching tile_z cells along z (0: automatic). M2C_FP64 results do
  * not depend on the tiling (bitwise); M2C_MIXED results agree to FP32 rounding
- * (FP32 multiply-adds may be contracted differently in the code that opens a
- * z-chunk and in the kernels of other tile heights). Default: the
+ * (the present kernels write their roundings out and gave the same bits for
+ * every tiling tried). A tile_z > 0 is taken as it is. Default: the
  * rows (8, or 4 for M2C_FP64 where 8 give too few tiles) and tile_z with the
  * smaller estimated time for the grid's size: short tiles that give every SM work
  * on a small grid, longer ones on a large grid. */
